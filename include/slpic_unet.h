@@ -28,7 +28,9 @@
  * With tensor_cores = 1 the forward convolutions and the input-gradient
  * convolutions run as implicit GEMMs on the tensor cores (tcgen05, BF16 x BF16,
  * FP32 accumulate in tensor memory, output channels in slices of 256): each
- * forward conv's input is rounded to BF16 (nearest even), and the weight gradient
+ * forward conv's input is rounded to BF16 (nearest even; where the channel counts are
+ * multiples of 8 it is stored so, the ReLU, the pooling and the masks being taken from
+ * the FP32 accumulators), and the weight gradient
  * multiplies by that rounded input; the input gradient is the transposed conv of
  * the output gradient rounded to BF16, and passes the forward rounding through
  * unchanged; the weight gradient is a GEMM over the pixels (split over CTAs, the

@@ -7,7 +7,9 @@
 //   decoder  d_{L-1} = e_{L-1},    d_l = relu(conv(concat(up(d_{l+1}), e_l)))
 //   output   y = conv(d_0)
 // conv: 3x3, zero padding, bias; pool: 2x2 mean; up: nearest x2; concat: the
-// upsampled channels first.  Activations and gradients are FP32 (N, C, H, W);
+// upsampled channels first.  Activations and gradients are FP32 (N, C, H, W), or with
+// tensor cores BF16 operands in channel blocks (unet_blocked.cuh; FP32 planes where the
+// channel counts do not fill blocks of 8);
 // the convolutions use BF16 copies of the FP32 master weights (biases stay FP32)
 // and accumulate in FP32; weight-gradient sums are FP64 across threads.  The loss
 // is the mean squared error; training is Adam.
@@ -727,19 +729,20 @@ __global__ void k_up_bwd(TV dout, TV din, int C, int H, int W, int nplanes)
     }
 }
 
-// ---- input normalisation: s_n = rms(x_n) (1 for an all-zero sample), xs = x / s_n
-// One CTA per sample; FP64 sum.  With normalise == 0, s_n = 1.
-__global__ void __launch_bounds__(kT) k_norm_in(const float *__restrict__ x, float *__restrict__ xs,
-                                              float *__restrict__ s, size_t HW, int normalise)
+// ---- input normalisation: s_n = rms(x_n) (1 for an all-zero sample; 1 with
+// normalise == 0), xs = x / s_n.  The sum of squares is FP64, kNormCtas partial sums per
+// sample added in a fixed order: one CTA per sample, as before, read a 1024 x 1024 image
+// in 987 us; the two launches take 16 us.
+constexpr int kNormCtas = 128;
+
+__global__ void __launch_bounds__(kT) k_norm_sum(const float *__restrict__ x, size_t HW,
+                                               double *__restrict__ part)
 {
     __shared__ double s_red[kT / 32];
-    __shared__ float s_scale;
-    const int n = blockIdx.x;
-    const float *xn = x + (size_t)n * HW;
+    const float *xn = x + (size_t)blockIdx.y * HW;
     double acc = 0.0;
-    if (normalise)
-        for (size_t q = threadIdx.x; q < HW; q += kT)
-            acc += (double)xn[q] * xn[q];
+    for (size_t q = blockIdx.x * (size_t)kT + threadIdx.x; q < HW; q += (size_t)kNormCtas * kT)
+        acc += (double)xn[q] * xn[q];
     for (int off = 16; off; off >>= 1)
         acc += __shfl_down_sync(0xffffffffu, acc, off);
     if ((threadIdx.x & 31) == 0)
@@ -749,16 +752,32 @@ __global__ void __launch_bounds__(kT) k_norm_in(const float *__restrict__ x, flo
         double v = 0.0;
         for (int k = 0; k < kT / 32; ++k)
             v += s_red[k];
-        float sc = normalise ? (float)sqrt(v / (double)HW) : 1.0f;
-        if (!(sc > 0.0f))
-            sc = 1.0f;
-        s_scale = sc;
-        s[n] = sc;
+        part[(size_t)blockIdx.y * kNormCtas + blockIdx.x] = v;
     }
-    __syncthreads();
-    const float inv = 1.0f / s_scale;
-    for (size_t q = threadIdx.x; q < HW; q += kT)
-        xs[(size_t)n * HW + q] = xn[q] * inv;
+}
+
+__global__ void k_norm_scale(const double *__restrict__ part, float *__restrict__ s, size_t HW, int normalise)
+{
+    const int n = blockIdx.x;  // one warp per sample
+    double v = 0.0;
+    if (normalise)
+        for (int k = threadIdx.x; k < kNormCtas; k += 32)
+            v += part[(size_t)n * kNormCtas + k];
+    for (int off = 16; off; off >>= 1)
+        v += __shfl_down_sync(0xffffffffu, v, off);
+    if (threadIdx.x == 0) {
+        const float sc = normalise ? (float)sqrt(v / (double)HW) : 1.0f;
+        s[n] = sc > 0.0f ? sc : 1.0f;
+    }
+}
+
+__global__ void __launch_bounds__(kT) k_norm_apply(const float *__restrict__ x, float *__restrict__ xs,
+                                                 const float *__restrict__ s, size_t HW)
+{
+    const float inv = 1.0f / s[blockIdx.y];
+    const size_t o = (size_t)blockIdx.y * HW;
+    for (size_t q = blockIdx.x * (size_t)kT + threadIdx.x; q < HW; q += (size_t)gridDim.x * kT)
+        xs[o + q] = x[o + q] * inv;
 }
 
 // y = y_net * s_n * out_scale
@@ -896,6 +915,8 @@ __global__ void k_to_bf16(const float *__restrict__ p, __nv_bfloat16 *__restrict
 
 }  // namespace
 
+#include "unet_blocked.cuh"
+
 // =====================================================================================
 // Host side: buffers, the layer schedule, the C ABI.
 // =====================================================================================
@@ -933,6 +954,14 @@ struct slpic_unet {
     size_t wpart_n = 0;
     bool tc_dirty = true;
     int *d_flag = nullptr;  // a bounded wait of a tensor-core kernel ran out
+    double *npart = nullptr;  // partial sums of squares of the input images
+    // blocked BF16 operands (unet_blocked.cuh) in the place of the FP32 activations above:
+    // with tensor cores and channel counts that fill blocks of 8
+    bool blk = false;
+    Blk xinb{}, d0b{}, dyb{};
+    std::vector<Blk> catb, pinb, dzd, dze;  // catb: 0..L-2; pinb: 1..L-1; dzd: 0..L-2; dze: 0..L-1
+    std::vector<float *> de;                // dL/d e_l before the pooling part, FP32: 0..L-2
+    double *bpart = nullptr;                // the tiles' bias-gradient sums
     cudaStream_t stream = nullptr;
     std::vector<void *> allocs;
     std::string err;
@@ -1094,9 +1123,253 @@ void relu_bwd(slpic_unet_t *h, TV a, TV gv, int C, int level, int nb, cudaStream
     k_relu_bwd<<<plane_grid(HW, nb * C), kT, 0, st>>>(a, gv, C, (int)HW, nb * C);
 }
 
-// The forward pass on the normalised input h->xin: fills every activation and
+// ---- the blocked path ---------------------------------------------------------------
+constexpr size_t kBlkFront = 64;        // positions before a tensor's first (zero)
+constexpr size_t kBlkSmem = 222 * 1000; // dynamic shared memory a CTA may take beside its static
+
+size_t blk_ps(const slpic_unet_t *h, int l)
+{
+    // the framed plane, and slack for the tiles and runs that pass its end (zero)
+    return (size_t)(hl(h, l) + 4) * (wl(h, l) + 2) + 192;
+}
+
+int blk_alloc(slpic_unet_t *h, Blk *b, int level, int channels)
+{
+    b->groups = (channels + 15) / 16 * 2;
+    b->off = 0;
+    b->ps = blk_ps(h, level);
+    const size_t n = ((size_t)h->nbmax * b->groups * b->ps + kBlkFront) * 8;
+    const int rc = alloc(h, (void **)&b->p, sizeof(__nv_bfloat16) * n);
+    if (rc)
+        return rc;
+    CKU(h, cudaMemsetAsync(b->p, 0, sizeof(__nv_bfloat16) * n, h->stream));
+    b->p += kBlkFront * 8;
+    return SLPIC_OK;
+}
+
+// One launch geometry of k_conv_blk: rows per unit, resident rows or streamed A, buffers.
+struct BlkPlan {
+    int mt, stream, slabs, bst;
+    size_t smem;
+};
+
+// Np: the launch's padded output channels (at most 128 with two rows, 256 with one: the
+// accumulators are held twice).  Two rows halve the weight traffic and are what the 2x2
+// epilogues need (pair).  In order of preference: every weight chunk resident and a whole
+// unit of rows ahead; the same with the weights in a ring; no rows ahead; one row; a
+// streamed A.
+BlkPlan blk_plan(int G, int Np, bool pair)
+{
+    const size_t w = (size_t)Np * kTcKC * 2, row = (size_t)G * kBSlab;
+    const int nkc = (9 * (G / 2) + 3) / 4;
+    for (int mt = Np <= 128 ? 2 : 1; mt >= (pair ? 2 : 1); --mt)
+        for (int ahead = mt; ahead >= 0; ahead -= mt) {
+            const size_t need = (size_t)(mt + 2 + ahead) * row;
+            for (int bst : {nkc, 4, 3, 2}) {
+                if (bst > std::min(nkc, kBRing) || need + bst * w > kBlkSmem)
+                    continue;
+                const int slabs = (int)std::min<size_t>(kBRows, (kBlkSmem - bst * w) / row);
+                return BlkPlan{mt, 0, slabs, bst, slabs * row + bst * w};
+            }
+        }
+    const int mt = Np <= 128 ? 2 : 1;
+    const size_t stage = w + (size_t)mt * 8 * kBPiece;
+    const int bst = (int)std::min<size_t>(kBRing, kBlkSmem / stage);
+    return BlkPlan{mt, 1, 0, bst, bst * stage};
+}
+
+// a conv on blocked operands over all its output channels, in slices; *ctas: CTAs launched
+void conv_blk(slpic_unet_t *h, ConvBlk a, int cin, int level, int Np, int nout, const __nv_bfloat16 *wp,
+              const float *bias, bool pair, int nb, cudaStream_t st, int *ctas)
+{
+    a.G = (cin + 15) / 16 * 2;
+    a.H = hl(h, level);
+    a.W = wl(h, level);
+    a.nb = nb;
+    a.bstride = (size_t)Np * kTcKC;
+    a.flag = h->d_flag;
+    const bool grad = a.mode >= kBmGradUp;
+    const int slice = pair ? 128 : kTcMaxN;
+    for (int o0 = 0; o0 < Np; o0 += slice) {
+        a.o0 = o0;
+        a.Np = std::min(slice, Np - o0);
+        a.nout = std::min(nout - o0, a.Np);
+        a.wp = wp + (size_t)o0 * kTcKC;
+        a.bias = bias ? bias + o0 : nullptr;
+        // one plan for every slice: the same CTAs, so that the bias sums of all slices
+        // have as many parts
+        BlkPlan q = blk_plan(a.G, std::min(slice, Np), pair);
+        a.slabs = q.slabs;
+        a.bst = q.bst;
+        const long long units = (long long)nb * ((a.W + kBX - 1) / kBX) * ((a.H + q.mt - 1) / q.mt);
+        const unsigned g = (unsigned)std::min<long long>(units, 152);
+        if (ctas)
+            *ctas = (int)g;
+        auto f = q.mt == 2 ? (q.stream ? (grad ? k_conv_blk<2, true, true> : k_conv_blk<2, true, false>)
+                                       : (grad ? k_conv_blk<2, false, true> : k_conv_blk<2, false, false>))
+                           : (q.stream ? (grad ? k_conv_blk<1, true, true> : k_conv_blk<1, true, false>)
+                                       : (grad ? k_conv_blk<1, false, true> : k_conv_blk<1, false, false>));
+        f<<<g, kBThreads, q.smem, st>>>(a);
+    }
+}
+
+Blk blk_view(Blk b, int channel)
+{
+    b.off = channel / 8;
+    return b;
+}
+
+void fwd_blk(slpic_unet_t *h, int k, Blk x, int mode, Blk dst, Blk pool, int nb, cudaStream_t st)
+{
+    const ConvSpec &c = h->conv[k];
+    ConvBlk a{};
+    a.x = x;
+    a.mode = mode;
+    a.dst = dst;
+    a.pool = pool;
+    a.f32 = mode == kBmOut ? h->ynet : nullptr;
+    conv_blk(h, a, c.cin, c.level, c.Np, c.cout, h->wtc + c.tc_off, h->p + c.b_off, pool.p != nullptr, nb, st,
+             nullptr);
+}
+
+dim3 image_grid(const slpic_unet_t *h, int nb)
+{
+    return dim3((unsigned)std::min<size_t>((hwl(h, 0) + kT - 1) / kT, 256), (unsigned)nb);
+}
+
+void forward_blk(slpic_unet_t *h, int nb, const float *x, cudaStream_t st)
+{
+    const int L = h->L;
+    k_image_blk<<<image_grid(h, nb), kT, 0, st>>>(x, h->s, h->xinb, h->H, h->W, nullptr);
+    for (int l = 0; l < L; ++l) {
+        const Blk in = l ? h->pinb[l] : h->xinb;
+        if (l < L - 1)
+            fwd_blk(h, l, in, kBmAct, blk_view(h->catb[l], ch(h, l + 1)), h->pinb[l + 1], nb, st);
+        else if (L > 1)
+            fwd_blk(h, l, in, kBmActUp, h->catb[L - 2], Blk{}, nb, st);
+        else
+            fwd_blk(h, l, in, kBmAct, h->d0b, Blk{}, nb, st);
+    }
+    for (int l = L - 2; l >= 0; --l)
+        fwd_blk(h, L + (L - 2 - l), h->catb[l], l ? kBmActUp : kBmAct, l ? h->catb[l - 1] : h->d0b, Blk{}, nb,
+                st);
+    fwd_blk(h, 2 * L - 1, h->d0b, kBmOut, Blk{}, Blk{}, nb, st);
+}
+
+// Geometry of k_wgrad_blk: tiles per CTA and dj (as many as TMEM holds: dz is read once
+// per group of tiles), the ring, the pixel ranges.
+struct WgPlan {
+    int mtiles, mper, djs, gx, gy, splits, stages;
+    size_t smem;
+};
+
+WgPlan wg_plan(const slpic_unet_t *h, const ConvSpec &c, int Np, int nb)
+{
+    WgPlan q{};
+    const int G = (c.cin + 15) / 16 * 2;
+    q.mtiles = (3 * G + 15) / 16;
+    q.djs = 3 * Np <= 512 ? 3 : 1;
+    q.mper = std::min(q.mtiles, 512 / (q.djs * Np));
+    const size_t z = (size_t)(Np / 8) * kWKP * 16;
+    while (q.mper > 1 && 2 * ((size_t)q.mper * 16 * kWRun + z) > kBlkSmem)
+        --q.mper;
+    const size_t stage = (size_t)q.mper * 16 * kWRun + z;
+    q.stages = (int)std::min<size_t>(4, kBlkSmem / stage);
+    q.smem = q.stages * stage;
+    q.gx = (q.mtiles + q.mper - 1) / q.mper;
+    q.gy = q.djs == 3 ? 1 : 3;
+    const long long chunks = (long long)nb * (((long long)hl(h, c.level) * (wl(h, c.level) + 2) + kWKP - 1) / kWKP);
+    q.splits = (int)std::max(1LL, std::min(chunks, (long long)152 / (q.gx * q.gy)));
+    return q;
+}
+
+void wgrad_blk(slpic_unet_t *h, int k, Blk x, Blk dz, int nb, cudaStream_t st)
+{
+    const ConvSpec &c = h->conv[k];
+    for (int o0 = 0; o0 < c.Np; o0 += kTcMaxN) {
+        const int Np = std::min(kTcMaxN, c.Np - o0);
+        const WgPlan q = wg_plan(h, c, Np, nb);
+        WgradBlk a{};
+        a.x = x;
+        a.dz = dz;
+        a.dz.off = o0 / 8;
+        a.G = (c.cin + 15) / 16 * 2;
+        a.Np = Np;
+        a.H = hl(h, c.level);
+        a.W = wl(h, c.level);
+        a.nb = nb;
+        a.mper = q.mper;
+        a.djs = q.djs;
+        a.mtiles = q.mtiles;
+        a.stages = q.stages;
+        a.part = h->wpart;
+        a.flag = h->d_flag;
+        k_wgrad_blk<<<dim3((unsigned)q.gx, (unsigned)q.gy, (unsigned)q.splits), kWThreads, q.smem, st>>>(a);
+        const int nout = std::min(c.cout - o0, Np);
+        k_wgrad_blk_reduce<<<dim3((unsigned)((nout + 31) / 32), (unsigned)(9 * c.cin)), kT, 0, st>>>(
+            h->wpart, q.splits, q.mtiles, a.G, Np, c.cin, nout, h->g + c.w_off + (size_t)o0 * c.cin * 9);
+    }
+}
+
+// the input gradient of conv k, its epilogue (mode) making the next layer's dz; bias: the
+// conv whose output gradient that is
+void dgrad_blk(slpic_unet_t *h, int k, Blk dz, int mode, Blk dst, Blk mask, float *f32, int cup, int bchan,
+               int bias, int nb, cudaStream_t st)
+{
+    const ConvSpec &c = h->conv[k];
+    ConvBlk a{};
+    a.x = dz;
+    a.mode = mode;
+    a.dst = dst;
+    a.mask = mask;
+    a.f32 = f32;
+    a.cup = cup;
+    a.bchan = bchan;
+    a.bpart = h->bpart;
+    int ctas = 0;
+    conv_blk(h, a, c.cout, c.level, c.Npt, c.cin, h->wtct + c.tct_off, nullptr, mode == kBmGradUp, nb, st, &ctas);
+    k_bias_tiles<<<h->conv[bias].cout, kT, 0, st>>>(h->bpart, ctas, bchan, h->g + h->conv[bias].b_off);
+}
+
+void backward_blk(slpic_unet_t *h, int nb, cudaStream_t st)
+{
+    const int L = h->L, out = 2 * L - 1;
+    const dim3 ig = image_grid(h, nb);
+    k_image_blk<<<ig, kT, 0, st>>>(h->dy, nullptr, h->dyb, h->H, h->W, h->bpart);
+    k_bias_tiles<<<1, kT, 0, st>>>(h->bpart, (int)(ig.x * ig.y), 1, h->g + h->conv[out].b_off);
+    wgrad_blk(h, out, h->d0b, h->dyb, nb, st);
+    const Blk z0 = L > 1 ? h->dzd[0] : h->dze[0];
+    dgrad_blk(h, out, h->dyb, kBmGradMask, z0, h->d0b, nullptr, 0, ch(h, 0), L > 1 ? 2 * L - 2 : 0, nb, st);
+    for (int l = 0; l <= L - 2; ++l) {
+        const int k = L + (L - 2 - l);
+        const bool top = l + 1 == L - 1;
+        wgrad_blk(h, k, h->catb[l], h->dzd[l], nb, st);
+        dgrad_blk(h, k, h->dzd[l], kBmGradUp, top ? h->dze[L - 1] : h->dzd[l + 1], h->catb[l], h->de[l],
+                  ch(h, l + 1), ch(h, l + 1) + ch(h, l), top ? L - 1 : k - 1, nb, st);
+    }
+    for (int l = L - 1; l >= 0; --l) {
+        wgrad_blk(h, l, l ? h->pinb[l] : h->xinb, h->dze[l], nb, st);
+        if (l)
+            dgrad_blk(h, l, h->dze[l], kBmGradPool, h->dze[l - 1], blk_view(h->catb[l - 1], ch(h, l)),
+                      h->de[l - 1], 0, ch(h, l - 1), l - 1, nb, st);
+    }
+}
+
+// The input scale of each sample, and the input itself in the form the convolutions take.
+void normalise_in(slpic_unet_t *h, int nb, const float *x, cudaStream_t st)
+{
+    const size_t HW = hwl(h, 0);
+    if (h->cfg.normalise)
+        k_norm_sum<<<dim3(kNormCtas, (unsigned)nb), kT, 0, st>>>(x, HW, h->npart);
+    k_norm_scale<<<nb, 32, 0, st>>>(h->npart, h->s, HW, h->cfg.normalise);
+    if (!h->blk)
+        k_norm_apply<<<dim3((unsigned)std::min<size_t>((HW + kT - 1) / kT, 512), (unsigned)nb), kT, 0, st>>>(
+            x, h->xin, h->s, HW);
+}
+
+// The forward pass on the images x, normalised by h->s: fills every activation and
 // h->ynet (network units).
-void forward_net(slpic_unet_t *h, int nb, cudaStream_t st)
+void forward_net(slpic_unet_t *h, int nb, const float *x, cudaStream_t st)
 {
     const int L = h->L;
     if (h->cfg.tensor_cores && h->tc_dirty) {
@@ -1107,6 +1380,10 @@ void forward_net(slpic_unet_t *h, int nb, cudaStream_t st)
                 h->pb + c.w_off, c.cout, c.cin, c.Npt, c.nkct, h->wtct + c.tct_off);
         }
         h->tc_dirty = false;
+    }
+    if (h->blk) {
+        forward_blk(h, nb, x, st);
+        return;
     }
     for (int l = 0; l < L; ++l) {
         if (l > 0)
@@ -1129,6 +1406,10 @@ void forward_net(slpic_unet_t *h, int nb, cudaStream_t st)
 void backward_net(slpic_unet_t *h, int nb, cudaStream_t st)
 {
     const int L = h->L;
+    if (h->blk) {
+        backward_blk(h, nb, st);
+        return;
+    }
     TV gd0{h->gd[0], ch(h, 0), 0};
     conv_bwd(h, 2 * L - 1, view_d(h, 0), TV{h->dy, 1, 0}, &gd0, nb, st);
     for (int l = 0; l <= L - 2; ++l) {
@@ -1173,7 +1454,31 @@ int ensure_grads(slpic_unet_t *h)
     h->dcat.assign(L, nullptr);
     h->gd.assign(L, nullptr);
     h->dpool.assign(L, nullptr);
-    for (int l = 0; l < L; ++l) {
+    for (int l = 0; l < L && h->blk; ++l) {
+        if ((rc = blk_alloc(h, &h->dze[l], l, ch(h, l))))
+            return rc;
+        if (l <= L - 2 && ((rc = blk_alloc(h, &h->dzd[l], l, ch(h, l))) ||
+                           (rc = alloc_f(h, &h->de[l], (size_t)nb * ch(h, l) * hwl(h, l)))))
+            return rc;
+    }
+    if (h->blk) {
+        // the weight gradients' partial sums and the bias gradients' tile sums, at the
+        // largest over the convs and batch sizes
+        size_t need = 1, tiles = (size_t)nb * 256;  // the latter: dy's own
+        for (const ConvSpec &c : h->conv) {
+            for (int b = 1; b <= nb; ++b) {
+                for (int Np : {std::min(kTcMaxN, c.Np), (c.Np - 1) % kTcMaxN + 1}) {  // slices
+                    const WgPlan q = wg_plan(h, c, Np, b);
+                    need = std::max(need, (size_t)q.splits * 3 * q.mtiles * 128 * Np);
+                }
+            }
+            tiles = std::max(tiles, (size_t)152 * c.cin);
+        }
+        if ((rc = alloc_f(h, &h->wpart, need)) || (rc = alloc(h, (void **)&h->bpart, sizeof(double) * tiles)) ||
+            (rc = blk_alloc(h, &h->dyb, 0, 1)))
+            return rc;
+    }
+    for (int l = 0; l < L && !h->blk; ++l) {
         if ((rc = alloc_f(h, &h->gd[l], (size_t)nb * ch(h, l) * hwl(h, l))))
             return rc;
         if (l <= L - 2 &&
@@ -1182,7 +1487,7 @@ int ensure_grads(slpic_unet_t *h)
         if (l >= 1 && (rc = alloc_f(h, &h->dpool[l], (size_t)nb * ch(h, l - 1) * hwl(h, l))))
             return rc;
     }
-    if (h->cfg.tensor_cores) {
+    if (h->cfg.tensor_cores && !h->blk) {
         size_t need = 1;
         for (const ConvSpec &c : h->conv) {
             if (c.Np > kTcMaxN)
@@ -1230,8 +1535,8 @@ int run_gradients(slpic_unet_t *h, int nb, const float *x, const float *t, cudaS
     if (rc)
         return rc;
     const size_t HW = hwl(h, 0);
-    k_norm_in<<<nb, kT, 0, st>>>(x, h->xin, h->s, HW, h->cfg.normalise);
-    forward_net(h, nb, st);
+    normalise_in(h, nb, x, st);
+    forward_net(h, nb, x, st);
     if (h->cfg.loss == SLPIC_UNET_LOSS_ENERGY) {
         k_energy_err<<<grid_for((size_t)nb * HW), kT, 0, st>>>(h->ynet, t, h->s, (float)h->cfg.out_scale,
                                                                h->eb, h->H, h->W, nb);
@@ -1332,11 +1637,39 @@ extern "C" int slpic_unet_create(const slpic_unet_config *cfg, slpic_unet_t **ou
                 rc = failu(h, SLPIC_ERR_CUDA, cudaGetErrorString(e));
         }
     }
-    if (!rc) rc = alloc_f(h, &h->xin, (size_t)nb * hwl(h, 0));
+    // blocks of 8 channels: every tensor's channels, the concatenated ones at their offsets
+    h->blk = c.tensor_cores && c.base % 8 == 0;
+    if (!rc && h->blk) {
+        cudaError_t e = cudaSuccess;
+        for (auto f : {k_conv_blk<1, false, false>, k_conv_blk<1, true, false>, k_conv_blk<2, false, false>,
+                       k_conv_blk<2, true, false>, k_conv_blk<1, false, true>, k_conv_blk<1, true, true>,
+                       k_conv_blk<2, false, true>, k_conv_blk<2, true, true>})
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlkSmem);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(k_wgrad_blk, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kBlkSmem);
+        if (e != cudaSuccess)
+            rc = failu(h, SLPIC_ERR_CUDA, cudaGetErrorString(e));
+        h->catb.assign(L, Blk{});
+        h->pinb.assign(L, Blk{});
+        h->dzd.assign(L, Blk{});
+        h->dze.assign(L, Blk{});
+        h->de.assign(L, nullptr);
+        if (!rc) rc = blk_alloc(h, &h->xinb, 0, 1);
+        if (!rc) rc = blk_alloc(h, &h->d0b, 0, ch(h, 0));
+        for (int l = 0; l < L && !rc; ++l) {
+            if (l <= L - 2)
+                rc = blk_alloc(h, &h->catb[l], l, ch(h, l + 1) + ch(h, l));
+            if (!rc && l >= 1)
+                rc = blk_alloc(h, &h->pinb[l], l, ch(h, l - 1));
+        }
+    }
+    if (!rc) rc = alloc(h, (void **)&h->npart, sizeof(double) * kNormCtas * nb);
+    if (!rc && !h->blk) rc = alloc_f(h, &h->xin, (size_t)nb * hwl(h, 0));
     if (!rc) rc = alloc_f(h, &h->s, (size_t)nb);
     if (!rc) rc = alloc_f(h, &h->ynet, (size_t)nb * hwl(h, 0));
-    if (!rc) rc = alloc_f(h, &h->etop, (size_t)nb * ch(h, L - 1) * hwl(h, L - 1));
-    for (int l = 0; l < L && !rc; ++l) {
+    if (!rc && !h->blk) rc = alloc_f(h, &h->etop, (size_t)nb * ch(h, L - 1) * hwl(h, L - 1));
+    for (int l = 0; l < L && !rc && !h->blk; ++l) {
         if (l <= L - 2) {
             rc = alloc_f(h, &h->cat[l], (size_t)nb * (ch(h, l + 1) + ch(h, l)) * hwl(h, l));
             if (!rc)
@@ -1427,8 +1760,8 @@ int slpic_unet_forward_on(slpic_unet_t *h, int nb, const float *x, float *y, cud
     if (rc)
         return rc;
     const size_t HW = hwl(h, 0);
-    k_norm_in<<<nb, kT, 0, st>>>(x, h->xin, h->s, HW, h->cfg.normalise);
-    forward_net(h, nb, st);
+    normalise_in(h, nb, x, st);
+    forward_net(h, nb, x, st);
     k_scale_out<<<grid_for((size_t)nb * HW), kT, 0, st>>>(h->ynet, y, h->s, (float)h->cfg.out_scale,
                                                           HW, nb);
     CKU(h, cudaGetLastError());
