@@ -5,15 +5,23 @@
 //               -> x^{n+1} = x^n + beta v dt -> walls -> FP64 CIC deposit of
 //               rho^{n+1} (global double atomics) -> survivors packed into the
 //               other buffer
-//   k_inject64  one CTA: source particles (FP64) appended and deposited; bookkeeping
-//   k_field64   one CTA: rho = sum_s q_s n_s, Poisson by FP64 prefix sums, E
+//   k_close64   one CTA: source particles (FP64) appended and deposited, bookkeeping;
+//               rho = sum_s q_s n_s, Poisson by FP64 prefix sums, E
 //
 // The velocity push solves the same equation as the mixed-precision library: with
 // w the velocity component along a, D = |v_perp|^2 and A = |a|, the time needed to
 // go from w_a to w is [H(w) - H(w_a)] / A with H(w) = int_0^w dw'/beta(sqrt(w'^2+D))
 // in closed form (int sqrt(w^2+D) dw = (w sqrt(w^2+D) + D asinh(w/sqrt D))/2), and
-// the new w solves H(w) = H(w_a) + A dt by Newton kept inside the bracket
-// [w_a, w_a + A dt] (H' = 1/beta >= 1).
+// the new w solves H(w) = H(w_a) + A dt.  Most particles need no iteration: inside the
+// band all step the push is the leapfrog, and where the step is small against the speed
+// the equation is reverted as a series (push_series64).  The rest are solved by Newton
+// kept inside the bracket [w_a, w_a + A dt] (H' = 1/beta >= 1), from an FP32 root.
+//
+// GB300's FP64 pipe has two lanes an SM, so the FP64 instructions of the push set the
+// time: each evaluation of H is some 150 of them, and Newton from the end of the bracket
+// took about five of them for every particle out of the band (51,200 particles on 256
+// cells: the particle kernel 819 us a step, now 46).
+#include <algorithm>
 #include <cmath>
 #include <string>
 #include <vector>
@@ -30,8 +38,10 @@ void set_create_error(const std::string &msg);              // api.cu
 namespace slpic64 {
 
 constexpr int kMaxS = SLPIC_MAX_SPECIES;
-constexpr int kThreads = 256;
-constexpr int kItems = 4;
+constexpr int kThreads = 128;
+// One particle per thread and tile: with four, 51,200 particles made 50 CTAs on 152 SMs,
+// and the FP64 pipe hides the latency of one.
+constexpr int kItems = 1;
 constexpr int kTile = kThreads * kItems;
 constexpr int kWarps = kThreads / 32;
 constexpr int kFieldThreads = 1024;
@@ -82,47 +92,108 @@ __device__ __forceinline__ double F64(double w, double D)
     return 0.5 * (w * sqrt(w * w + D) + D * asinh(w / sqrt(D)));
 }
 
-__device__ double H64(int kind, double w, double D, double v0)
+// H along one line: D and what of H does not depend on w
+struct Line64 {
+    int kind;
+    double D, v0, W0, F0;  // Heaviside with a band (band = true): its edge and F(W0)
+    bool band;
+};
+
+__device__ __forceinline__ Line64 line64(int kind, double D, double v0)
 {
-    if (kind == SLPIC_BETA_ONE)
-        return w;
-    if (kind == SLPIC_BETA_RELATIVISTIC)
-        return F64(w, D + v0 * v0) / v0;
-    if (D < v0 * v0) {
-        const double W0 = sqrt(v0 * v0 - D);
-        if (fabs(w) <= W0)
-            return w;
-        const double s = w < 0.0 ? -1.0 : 1.0;
-        return s * (W0 + (F64(fabs(w), D) - F64(W0, D)) / v0);
+    Line64 l{kind, D, v0, 0.0, 0.0, false};
+    if (kind == SLPIC_BETA_RELATIVISTIC) {
+        l.D = D + v0 * v0;
+    } else if (D < v0 * v0) {
+        l.band = true;
+        l.W0 = sqrt(v0 * v0 - D);
+        l.F0 = F64(l.W0, D);
     }
-    return F64(w, D) / v0;
+    return l;
 }
 
-__device__ __forceinline__ double inv_beta64(int kind, double w, double D, double v0)
+__device__ __forceinline__ double H64(const Line64 &l, double w)
 {
-    return 1.0 / beta64(kind, sqrt(w * w + D), v0);
+    if (!l.band)
+        return F64(w, l.D) / l.v0;
+    if (fabs(w) <= l.W0)
+        return w;
+    const double s = w < 0.0 ? -1.0 : 1.0;
+    return s * (l.W0 + (F64(fabs(w), l.D) - l.F0) / l.v0);
 }
 
-// new velocity component along x after one step of the push with a = (ax, 0, 0)
-__device__ double push64(int kind, double ux, double uy, double uz, double ax, double dt, double v0)
+// The same H in FP32, for the start of the iteration only.
+__device__ __forceinline__ float F32(float w, float D)
 {
-    if (kind == SLPIC_BETA_ONE || ax == 0.0)
-        return ux + ax * dt;  // beta == 1 (or no force): plain leapfrog
-    const double A = fabs(ax), sg = ax > 0.0 ? 1.0 : -1.0;
-    const double wa = sg * ux, D = uy * uy + uz * uz, budget = A * dt;
-    const double Ha = H64(kind, wa, D, v0), T = Ha + budget;
+    if (D <= 0.0f)
+        return 0.5f * w * fabsf(w);
+    return 0.5f * (w * sqrtf(w * w + D) + D * asinhf(w * rsqrtf(D)));
+}
+
+// A root of H(w) = H(wa) + budget in [wa, wa + budget] to FP32 accuracy (some 20 FP32
+// instructions an evaluation, beside 150 on the narrow FP64 pipe).
+__device__ __forceinline__ float seed32(const Line64 &l, float wa, float budget)
+{
+    const float D = (float)l.D, v0 = (float)l.v0, W0 = (float)l.W0, F0 = (float)l.F0;
+    auto H = [&](float w) {
+        if (!l.band)
+            return F32(w, D) / v0;
+        if (fabsf(w) <= W0)
+            return w;
+        const float t = W0 + (F32(fabsf(w), D) - F0) / v0;
+        return w < 0.0f ? -t : t;
+    };
+    const float T = H(wa) + budget;
+    float lo = wa, hi = wa + budget, w = hi;
+    for (int it = 0; it < 24; ++it) {
+        const float g = H(w) - T;
+        if (g > 0.0f)
+            hi = w;
+        else
+            lo = w;
+        const float slope = (l.band && fabsf(w) <= W0) ? 1.0f : sqrtf(w * w + D) / v0;
+        float wn = w - g / slope;
+        if (!(wn > lo && wn < hi))
+            wn = 0.5f * (lo + hi);
+        const bool small = fabsf(wn - w) <= 3e-7f * fmaxf(fabsf(w), budget);
+        w = wn;
+        if (small)
+            break;
+    }
+    return w;
+}
+
+// w after the step along +a, by safeguarded Newton (out of line: few particles)
+__device__ __noinline__ double push_newton64(int kind, double wa, double D, double budget, double v0)
+{
+    const Line64 l = line64(kind, D, v0);
+    const double Ha = H64(l, wa), T = Ha + budget;
     // H is evaluated to a few ulp of its size: below that the residual is noise
     const double gtol = 8.0 * 2.220446049250313e-16 * (fabs(Ha) + budget);
     double lo = wa, hi = wa + budget, w = hi;
+    const double w0 = (double)seed32(l, (float)wa, (float)budget);
+    if (w0 > lo && w0 < hi)  // else (or not a number: beyond FP32's range) from the end
+        w = w0;
     for (int it = 0; it < 60; ++it) {
-        const double g = H64(kind, w, D, v0) - T;
+        const double g = H64(l, w) - T;
         if (fabs(g) <= gtol)
             break;
         if (g > 0.0)
             hi = w;
         else
             lo = w;
-        double wn = w - g / inv_beta64(kind, w, D, v0);
+        const double r = sqrt(w * w + l.D), ib = (l.band && r <= v0) ? 1.0 : r / v0;  // H' = 1/beta
+        const double dw = g / ib;
+        // Halley's step where H'' = w/(r v0) holds on both sides of it (off the band's
+        // edge): its error is of third order, below an ulp of r after so short a step, so
+        // that the FP32 root is followed by one evaluation
+        if (fabs(dw) <= 4e-6 * r && !(l.band && fabs(fabs(w) - l.W0) <= 4.0 * fabs(dw))) {
+            const double h2 = (l.band && r <= v0) ? 0.0 : w / (r * r);  // H''/H'
+            const double wh = w - dw * (1.0 + 0.5 * dw * h2);
+            w = fmin(fmax(wh, lo), hi);
+            break;
+        }
+        double wn = w - dw;
         if (!(wn > lo && wn < hi))
             wn = 0.5 * (lo + hi);
         const bool small = fabs(wn - w) <= 1e-14 * fmax(fabs(w), budget);
@@ -130,7 +201,61 @@ __device__ double push64(int kind, double ux, double uy, double uz, double ax, d
         if (small)
             break;
     }
-    return sg * w;
+    return w;
+}
+
+// Reversion of int_0^z sqrt(1 + 2 om s + s^2) ds = k, i.e. of the step's equation on a
+// smooth piece with z = (w - wa)/ra, ra = sqrt(wa^2 + D), om = wa/ra, k = y/ra^2:
+//   z = k (1 + b2 k + b3 k^2 + ... + b10 k^9),
+// the coefficients from z'^2 (1 + 2 om z + z^2) = 1, order by order (computer algebra).
+// Against 40-digit roots over om in [-1, 1] the truncation is below 4e-18 ra at k = 0.02
+// and falls as k^11: a thirtieth of an FP64 ulp of the speed.
+constexpr double kSeries64 = 0.02;
+
+__device__ __forceinline__ double push_series64(double om, double k)
+{
+    const double o2 = om * om, k2 = k * k;
+    const double b3 = fma(2.0 / 3.0, o2, -1.0 / 6.0);
+    const double b5 = fma(fma(7.0 / 3.0, o2, -47.0 / 30.0), o2, 13.0 / 120.0);
+    const double b7 = fma(fma(fma(104.0 / 9.0, o2, -187.0 / 15.0), o2, 43.0 / 14.0), o2, -493.0 / 5040.0);
+    const double b9 = fma(fma(fma(fma(5434.0 / 81.0, o2, -16115.0 / 162.0), o2, 82247.0 / 1890.0), o2,
+                              -256061.0 / 45360.0), o2, 37369.0 / 362880.0);
+    const double d4 = fma(-7.0 / 6.0, o2, 13.0 / 24.0);
+    const double d6 = fma(fma(-91.0 / 18.0, o2, 797.0 / 180.0), o2, -493.0 / 720.0);
+    const double d8 = fma(fma(fma(-247.0 / 9.0, o2, 4219.0 / 120.0), o2, -20147.0 / 1680.0), o2,
+                          37369.0 / 40320.0);
+    const double d10 = fma(fma(fma(fma(-13585.0 / 81.0, o2, 457589.0 / 1620.0), o2, -407891.0 / 2700.0), o2,
+                               12760871.0 / 453600.0), o2, -4732249.0 / 3628800.0);
+    const double ev = fma(fma(fma(fma(b9, k2, b7), k2, b5), k2, b3), k2, 1.0);
+    const double od = fma(fma(fma(fma(d10, k2, d8), k2, d6), k2, d4), k2, -0.5) * k;
+    return fma(om, od, ev);
+}
+
+// new velocity component along x after one step of the push with a = (ax, 0, 0)
+__device__ __forceinline__ double push64(int kind, double ux, double uy, double uz, double ax, double dt,
+                                         double v0)
+{
+    if (kind == SLPIC_BETA_ONE || ax == 0.0)
+        return ux + ax * dt;  // beta == 1 (or no force): plain leapfrog
+    const double A = fabs(ax), sg = ax > 0.0 ? 1.0 : -1.0;
+    const double wa = sg * ux, D = uy * uy + uz * uz, budget = A * dt, v02 = v0 * v0;
+    double Ds = D;
+    if (kind == SLPIC_BETA_HEAVISIDE) {
+        const double wb = wa + budget, sa = wa * wa + D, sb = wb * wb + D;
+        // |v| is convex along the line: both ends in the band, the whole step is
+        if (sa <= v02 && sb <= v02)
+            return sg * wb;
+        // a smooth piece: no band on the line, or the step starts above it, or ends
+        // below it even at leapfrog speed
+        if (D < v02 && !((wa >= 0.0 && sa >= v02) || (wb <= 0.0 && sb >= v02)))
+            return sg * push_newton64(kind, wa, D, budget, v0);
+    } else {
+        Ds = D + v02;
+    }
+    const double inv = rsqrt(wa * wa + Ds), yr = budget * v0 * inv, kap = yr * inv;
+    if (!(kap <= kSeries64))
+        return sg * push_newton64(kind, wa, D, budget, v0);
+    return sg * fma(yr, push_series64(wa * inv, kap), wa);
 }
 
 // ---- counter-based SplitMix64 (Steele, Lea & Flood, OOPSLA 2014) ------------------
@@ -199,9 +324,11 @@ __global__ void __launch_bounds__(kThreads) k_step64(P64 p)
                                     sp.v0);
             double xn = x[k] + b * vx[k] * p.dt;
             if (p.periodic) {
-                xn -= p.L * floor(xn / p.L);
-                if (xn >= p.L)
-                    xn -= p.L;
+                if (xn < 0.0 || xn >= p.L) {
+                    xn -= p.L * floor(xn / p.L);
+                    if (xn >= p.L)
+                        xn -= p.L;
+                }
             } else if (xn < 0.0 || xn >= p.L) {
                 atomicAdd(&s_abs[xn < 0.0 ? 0 : 1], 1u);
                 live[k] = false;
@@ -228,7 +355,7 @@ __global__ void __launch_bounds__(kThreads) k_step64(P64 p)
         }
         __syncthreads();
         if (warp == 0) {
-            const int v = s_cnt[lane];
+            const int v = lane < kItems * kWarps ? s_cnt[lane] : 0;
             int incl = v;
 #pragma unroll
             for (int o = 1; o < 32; o <<= 1) {
@@ -236,7 +363,8 @@ __global__ void __launch_bounds__(kThreads) k_step64(P64 p)
                 if (lane >= o)
                     incl += y;
             }
-            s_cnt[lane] = incl - v;
+            if (lane < kItems * kWarps)
+                s_cnt[lane] = incl - v;
             const int tot = __shfl_sync(0xffffffffu, incl, 31);
             if (lane == 0)
                 s_base = tot ? atomicAdd(&p.st->count[s][P ^ 1], (unsigned long long)tot) : 0ULL;
@@ -283,8 +411,8 @@ __global__ void __launch_bounds__(kThreads) k_deposit64(P64 p)
     }
 }
 
-// source (the volume source of the library, in FP64) and bookkeeping; one CTA
-__global__ void __launch_bounds__(1024) k_inject64(P64 p)
+// source (the volume source of the library, in FP64) and bookkeeping, by one CTA
+__device__ void inject64(const P64 &p)
 {
     __shared__ long long s_k[kMaxS], s_base[kMaxS];
     __shared__ double s_frac[kMaxS];
@@ -421,9 +549,10 @@ __device__ double scan64(double v, double *s_w, double *total)
 // removing the mean of rho); phi_j = phi_0 + j D_0 - sum_{i<j} P_i;
 // E_j = -(D_{j-1} + D_j)/(2 dx), one-sided at the plates.  One CTA, each thread a
 // contiguous chunk of at most kMaxChunk nodes; the consumed deposit is cleared.
+// __ldcg: the deposits were made by atomics in L2, this CTA's own among them.
 constexpr int kMaxChunk = 64;
 
-__global__ void __launch_bounds__(kFieldThreads) k_field64(P64 p)
+__device__ void field64(const P64 &p)
 {
     __shared__ double s_w[32];
     const int N = p.N, nn = p.nn;
@@ -435,7 +564,7 @@ __global__ void __launch_bounds__(kFieldThreads) k_field64(P64 p)
         const int j = j0 + k;
         double r = 0.0;
         for (int s = 0; s < p.ns; ++s) {
-            r += p.q[s] * p.dens[(size_t)s * nn + j];
+            r += p.q[s] * __ldcg(p.dens + (size_t)s * nn + j);
             p.dens[(size_t)s * nn + j] = 0.0;
         }
         p.rho[j] = r;
@@ -494,6 +623,26 @@ __global__ void __launch_bounds__(kFieldThreads) k_field64(P64 p)
         for (int j = j0; j < j1; ++j)
             p.phi[j] -= pt / N;
     }
+}
+
+// mode 1: the end of a step (source, bookkeeping, field); 0: the field alone.  One launch
+// for both halves, with no more threads than the grid has nodes: the block scans' FP64
+// additions are what the kernel waits for, and idle warps would take their turns on the
+// pipe (256 nodes: 5.4 + 20.4 us as two launches of 1,024 threads).
+__global__ void __launch_bounds__(kFieldThreads) k_close64(P64 p, int mode)
+{
+    if (mode) {
+        inject64(p);
+        __threadfence();
+        __syncthreads();
+    }
+    field64(p);
+}
+
+int close_threads(const P64 &p, int mode)
+{
+    const int n = mode && p.src_mode != SLPIC_SRC_NONE ? 512 : 128;  // source particles too
+    return std::min(kFieldThreads, std::max(n, (p.nn + 31) / 32 * 32));
 }
 
 }  // namespace slpic64
@@ -699,7 +848,7 @@ extern "C" int slpic_fp64_prepare(slpic_fp64_t *h)
     P64 &p = h->p;
     CK64(h, cudaMemsetAsync(p.dens, 0, sizeof(double) * p.nn * p.ns, h->stream));
     k_deposit64<<<dim3(h->ctas, p.ns), kThreads, 0, h->stream>>>(p);
-    k_field64<<<1, kFieldThreads, 0, h->stream>>>(p);
+    k_close64<<<1, close_threads(p, 0), 0, h->stream>>>(p, 0);
     CK64(h, cudaGetLastError());
     return slpic_fp64_synchronize(h);
 }
@@ -712,8 +861,7 @@ extern "C" int slpic_fp64_step(slpic_fp64_t *h, int64_t nsteps)
     const size_t smem = sizeof(double) * (size_t)p.nn;
     for (int64_t k = 0; k < nsteps; ++k) {
         k_step64<<<dim3(h->ctas, p.ns), kThreads, smem, h->stream>>>(p);
-        k_inject64<<<1, 1024, 0, h->stream>>>(p);
-        k_field64<<<1, kFieldThreads, 0, h->stream>>>(p);
+        k_close64<<<1, close_threads(p, 1), 0, h->stream>>>(p, 1);
     }
     CK64(h, cudaGetLastError());
     return SLPIC_OK;
