@@ -48,10 +48,10 @@ constexpr int kItems = 4;                       // particles per thread per tile
 constexpr int kTile = kThreads * kItems;
 constexpr int kWarps = kThreads / 32;
 constexpr int kCompact2d = 16;                  // compacting step interval
-constexpr int kCgThreads = 256;
-constexpr int kBarGroup = 16;   // CTAs per first-level group of the grid barrier
-constexpr int kBarGroups = 64;  // first-level counters (CG grids up to 1,024 CTAs)
-constexpr long long kBarrierSpins = 1LL << 23;  // bounded grid-barrier wait (~1 s)
+constexpr int kCgVirtual = 256;  // threads of a virtual CTA of the CG: a unit of its sums
+constexpr int kCgThreads = 2 * kCgVirtual;
+constexpr int kCgMaxVirtual = 512;             // virtual CTAs (two per SM)
+constexpr long long kCgWaitCycles = 2000000000LL;  // bounded wait for the other CTAs (~1 s)
 constexpr long long kMaxTimedSteps2d = 4096;    // steps recorded by the kernel timing
 
 // A particle whose push needs the piece walk, listed by the in-place tile kernel
@@ -90,8 +90,6 @@ struct State2D {
     double cg_res;
     int cg_iters;
     int error;
-    unsigned bar_count, bar_gen;  // grid barrier of k_cg2d: root counter, generation
-    unsigned bar_group[kBarGroups];  // first-level counters of the grid barrier
 };
 
 struct Params2D {
@@ -111,7 +109,8 @@ struct Params2D {
     float2 *E;                // [nn] (Ex, Ey)
     double *phi, *r, *q;            // [nn] FP64: solution, standalone solve's rho, b
     float *fr, *fpA, *fpB, *fq, *fd;  // [nn] FP32 CG iterates, zero on the plate rows
-    double *part;             // [3][grid] per-CTA partial sums
+    double *part;             // [3][cg_v] the CG's partial sums, by turn (kCgEmpty: not there yet)
+    int cg_v;                 // virtual CTAs of the CG's sums
     State2D *st;
     // direct solver (SLPIC2D_SOLVER_FFT)
     int solver, log2nx;
@@ -994,77 +993,175 @@ __global__ void k_book2d(Params2D p, int compact)
 // everywhere and in every run.
 // ---------------------------------------------------------------------------------
 
-// Grid barrier for a cooperative launch (all CTAs co-resident), two levels: CTAs
-// arrive on the counter of their group of kBarGroup, the last of each group on the
-// root counter, and the last of all advances the generation the others wait on
-// (each counter is reset by its last arriver before the generation moves).  The
-// wait is bounded: past kBarrierSpins polls the kernel records SLPIC_ERR_TIMEOUT
-// and every CTA leaves at its next check.
-__device__ __forceinline__ bool grid_sync(State2D *st)
+// The CG's sums and barriers are one: a virtual CTA of kCgVirtual threads writes its
+// partial sum to its slot, and every CTA polls all slots and adds them itself, in one
+// fixed order (the same value everywhere and in every run).  That costs a write and a
+// read of L2; a barrier of counters (atomics by groups, a generation word, sleeps) and
+// then a read of the sums took 11 us a sum on 304 CTAs (now 6 at 250 x 241, 4 at 64 x 48).
+// Slots go by three turns: a CTA empties its slots of the next turn before it writes this
+// one's, when every CTA has passed the turn before and so read the one that used them.
+//
+// The order of the additions is that of cg_v CTAs of kCgVirtual threads, whatever is
+// launched (a tree over each warp's lanes, the warps in order, the same over the CTAs'
+// sums): CTAs of two virtual ones, and none for virtual CTAs without nodes, whose sums
+// are zero.  What a sum costs is FP64 latency (an addition is 110 cycles on an idle pipe
+// of 2 lanes an SM): the trees' levels are packed into as few warps as have pairs left,
+// and the scalar work that follows is thread 0's alone (then, below).
+constexpr unsigned long long kCgEmpty = ~0ULL;  // a NaN that no sum is stored as
+
+struct CgShared {
+    double v[kCgThreads], g[kCgVirtual];
+};
+
+struct CgSync {
+    CgShared *sh;
+    double *part;
+    int v;     // virtual CTAs
+    int turn;  // of the next sum
+    int *error;
+};
+
+// float -> double on the integer pipe (the conversion instruction takes the FP64 pipe);
+// zeros, subnormals, infinities and NaN by the instruction
+__device__ __forceinline__ double cg_double(float x)
 {
-    __shared__ int s_ok;
+    const unsigned u = __float_as_uint(x), e = u & 0x7F800000u;
+    if (e == 0u || e == 0x7F800000u)
+        return (double)x;
+    return __hiloint2double((int)((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + 0x38000000u)), (int)(u << 29));
+}
+
+// (float)(a / b), the FP64 quotient rounded to FP32, without the FP64 division's chain of
+// some 15 dependent instructions: the significands as pairs of floats, a quotient with a
+// correction good to 2^-43, rounded; the FP64 division where that lies within 2^-38 of
+// the middle between two floats (one quotient in 2^13), or where the operands or the
+// quotient leave the normal range.
+__device__ __forceinline__ float cg_quotient(double a, double b)
+{
+    const unsigned ah = (unsigned)__double2hiint(a), al = (unsigned)__double2loint(a);
+    const unsigned bh = (unsigned)__double2hiint(b), bl = (unsigned)__double2loint(b);
+    const int ea = (int)(ah >> 20), eb = (int)(bh >> 20);  // sign included: negative is out of range
+    const int e = ea - eb;
+    if (ea >= 1 && ea < 2047 && eb >= 1 && eb < 2047 && e > -120 && e < 120) {
+        // 1.m = hi + lo: 24 bits and the 29 below them
+        const float xh = __uint_as_float(0x3F800000u | ((ah & 0xFFFFFu) << 3) | (al >> 29));
+        const float yh = __uint_as_float(0x3F800000u | ((bh & 0xFFFFFu) << 3) | (bl >> 29));
+        const float xl = __fmul_rn((float)(al & 0x1FFFFFFFu), 0x1p-52f);
+        const float yl = __fmul_rn((float)(bl & 0x1FFFFFFFu), 0x1p-52f);
+        const float inv = __frcp_rn(yh);
+        const float q0 = __fmul_rn(xh, inv);
+        const float r = __fmaf_rn(-q0, yh, xh);  // exact
+        const float q1 = __fmul_rn(__fmaf_rn(-q0, yl, __fadd_rn(r, xl)), inv);
+        const float q = __fadd_rn(q0, q1);
+        const float d = __fsub_rn(q1, __fsub_rn(q, q0));  // the quotient is q + d
+        // the middles to q's neighbours lie half an ulp off (a quarter below a power of two)
+        const float ulp = q >= 1.0f ? 0x1p-23f : 0x1p-24f;
+        const float m = fabsf(d);
+        if (fabsf(__fsub_rn(m, 0.5f * ulp)) > 0x1p-38f && fabsf(__fsub_rn(m, 0.25f * ulp)) > 0x1p-38f && q > 0.5f)
+            return __fmul_rn(q, __uint_as_float((unsigned)(e + 127) << 23));
+    }
+    return (float)(a / b);
+}
+
+__device__ __forceinline__ void cg_release()
+{
+    asm volatile("fence.acq_rel.gpu;" ::: "memory");
+}
+__device__ __forceinline__ unsigned long long cg_acquire(const unsigned long long *a)
+{
+    unsigned long long v;
+    asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(a) : "memory");
+    return v;
+}
+__device__ __forceinline__ void cg_store(unsigned long long *a, unsigned long long v)
+{
+    asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(a), "l"(v) : "memory");
+}
+
+// The sum of v over all threads, given to then(sum) in every CTA's thread 0; also a
+// barrier of all CTAs, after which their writes before it are visible (read them through
+// L2) and what then() left in shared memory is.  False if a wait gave up.
+template <typename Then>
+__device__ __forceinline__ bool cg_sum(CgSync &sy, double v, Then then)
+{
+    // the second tree has its own array: another warp may be there while the first still
+    // reads the last level of its own
+    double *s_v = sy.sh->v, *s_g = sy.sh->g;
+    constexpr int kW = kCgThreads / 32, kVW = kCgVirtual / 32;  // warps, of them a virtual CTA's
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    unsigned long long *slots = reinterpret_cast<unsigned long long *>(sy.part);
+    // tree over the lanes of every warp: lane l of warp w at l kW + w, so that a level's
+    // pairs are threads next to one another
+    s_v[lane * kW + warp] = v;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        volatile unsigned *gen = &st->bar_gen;
-        const unsigned g = *gen;
-        __threadfence();
-        const unsigned grp = blockIdx.x / kBarGroup;
-        const unsigned ngrp = (gridDim.x + kBarGroup - 1) / kBarGroup;
-        const unsigned in_grp = min((unsigned)kBarGroup, gridDim.x - grp * kBarGroup);
-        bool last = false;
-        if (atomicAdd(&st->bar_group[grp], 1u) == in_grp - 1) {
-            st->bar_group[grp] = 0u;
-            __threadfence();
-            if (atomicAdd(&st->bar_count, 1u) == ngrp - 1) {
-                st->bar_count = 0u;
-                __threadfence();
-                atomicAdd(&st->bar_gen, 1u);
-                last = true;
-            }
+    double g = 0.0;
+#pragma unroll
+    for (int n = kCgThreads / 2; n >= 32; n >>= 1) {  // lanes l and l + n / kW
+        if (t < n) {
+            g = (n == kCgThreads / 2 ? s_v[t] : g) + s_v[t + n];
+            if (t >= n / 2 && n > 32)
+                s_v[t] = g;
         }
-        if (!last) {
-            long long spins = 0;
-            while (*gen == g) {
-                if (++spins > kBarrierSpins) {
-                    atomicCAS(&st->error, 0, SLPIC_ERR_TIMEOUT);
+        if (n > 32)
+            __syncthreads();
+    }
+    if (warp == 0) {
+        static_assert(kW == 16, "the last level's pairs are half a warp apart");
+        g += __shfl_down_sync(0xffffffffu, g, 16);  // lane w: the sum of warp w
+        double c = 0.0;
+#pragma unroll
+        for (int k = 0; k < kVW; ++k)
+            c += __shfl_sync(0xffffffffu, g, (lane & kVW) + k);
+        if (lane == 0 || lane == kVW) {
+            const int vcta = blockIdx.x * 2 + (lane ? 1 : 0), next = sy.turn == 2 ? 0 : sy.turn + 1;
+            cg_store(slots + next * sy.v + vcta, kCgEmpty);
+            cg_release();  // the CTA's writes (seen through the barriers) and the emptied slot
+            cg_store(slots + sy.turn * sy.v + vcta,
+                     isnan(c) ? 0x7FF8000000000000ULL : (unsigned long long)__double_as_longlong(c));
+        }
+    }
+    bool ok = true;
+    g = 0.0;
+    if (t < kCgVirtual) {
+        const long long t0 = clock64();
+        for (int b = t; b < (int)gridDim.x * 2; b += kCgVirtual) {
+            unsigned long long u;
+            while ((u = cg_acquire(slots + sy.turn * sy.v + b)) == kCgEmpty)
+                if (clock64() - t0 > kCgWaitCycles) {
+                    atomicCAS(sy.error, 0, SLPIC_ERR_TIMEOUT);
+                    ok = false;
                     break;
                 }
-                __nanosleep(64);
-            }
+            const double x = __longlong_as_double((long long)u);
+            g = b < kCgVirtual ? x : g + x;
         }
-        __threadfence();
-        // one decision per CTA, so that its threads leave or stay together
-        s_ok = *(volatile int *)&st->error != SLPIC_ERR_TIMEOUT;
+        s_g[lane * kVW + warp] = g;  // the same tree over the virtual CTAs' sums
+    }
+    sy.turn = sy.turn == 2 ? 0 : sy.turn + 1;
+    if (!__syncthreads_and(ok))
+        return false;
+#pragma unroll
+    for (int n = kCgVirtual / 2; n >= 32; n >>= 1) {
+        if (t < n) {
+            g = (n == kCgVirtual / 2 ? s_g[t] : g) + s_g[t + n];
+            if (t >= n / 2 && n > 32)
+                s_g[t] = g;
+        }
+        if (n > 32)
+            __syncthreads();
+    }
+    if (warp == 0) {
+        g += __shfl_down_sync(0xffffffffu, g, 16);
+        g += __shfl_down_sync(0xffffffffu, g, 8);
+        double c = 0.0;
+#pragma unroll
+        for (int k = 0; k < kVW; ++k)
+            c += __shfl_sync(0xffffffffu, g, k);
+        if (lane == 0)
+            then(c);
     }
     __syncthreads();
-    return s_ok != 0;
-}
-
-// block sum of v (FP64, fixed order), result valid in every thread
-__device__ __forceinline__ double block_sum(double v, double *s_red)
-{
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int o = 16; o; o >>= 1)
-        v += __shfl_down_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if (lane == 0)
-        s_red[warp] = v;
-    __syncthreads();
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w)
-        t += s_red[w];
-    return t;
-}
-
-// sum of the CTAs' partials, in CTA order
-__device__ __forceinline__ double grid_total(const double *part, double *s_red)
-{
-    double v = 0.0;
-    for (int b = threadIdx.x; b < (int)gridDim.x; b += blockDim.x)
-        v += __ldcg(part + b);
-    // fixed assignment of CTAs to threads and a fixed tree: the same in every CTA
-    return block_sum(v, s_red);
+    return true;
 }
 
 // Arrays written by other CTAs of the cooperative grid are read with __ldcg
@@ -1113,18 +1210,23 @@ __device__ __forceinline__ void store_E(const Params2D &p, int idx)
 // an update at every tenfold drop.  The solve ends when that true residual meets ||b - A phi|| <= rtol ||b||,
 // the figure reported.  FP64 arithmetic, narrow on this GPU, is left to the few
 // updates.
+//
+// Node t of the interior belongs to thread t modulo the virtual grid's threads, at most K
+// per thread, whose r, d, q and p stay in its registers: only the p and r that neighbours
+// read go to memory.  K = 0: any number, all in memory (fd, fq).
 constexpr double kUpdateDrop = 1e-1;
 
-__global__ void __launch_bounds__(kCgThreads) k_cg2d(Params2D p, int mode)
+template <int K>
+__global__ void __launch_bounds__(kCgThreads, 1) k_cg2d(const __grid_constant__ Params2D p, int mode)
 {
-    __shared__ double s_red[kCgThreads / 32];
     State2D *st = p.st;
     const int nx = p.nx, ny = p.ny, nn = p.nn;
     const int first = nx, last = ny * nx;  // interior nodes [first, last)
     const long long gtid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const long long gstride = (long long)gridDim.x * blockDim.x;
-    double *part0 = p.part, *part1 = p.part + gridDim.x, *part2 = p.part + 2 * gridDim.x;
+    const long long gstride = (long long)p.cg_v * kCgVirtual;
     double *b64 = p.q;  // right-hand side, kept for the true residuals
+    __shared__ CgShared s_sums;
+    CgSync sy{&s_sums, p.part, p.cg_v, 0, &st->error};
 
     // ---- b (FP64, interior rows; 0 on the plates) and ||b||^2; FP32 iterates zeroed
     double bb = 0.0;
@@ -1154,25 +1256,38 @@ __global__ void __launch_bounds__(kCgThreads) k_cg2d(Params2D p, int mode)
         p.fr[idx] = 0.0f;
         p.fpA[idx] = 0.0f;
         p.fpB[idx] = 0.0f;
-        p.fd[idx] = 0.0f;
+        if (K == 0)
+            p.fd[idx] = 0.0f;
     }
-    bb = block_sum(bb, s_red);
-    if (threadIdx.x == 0)
-        part0[blockIdx.x] = bb;
-    if (!grid_sync(st))
+    // thread 0's scalars (no other thread has them), and what it tells the others
+    double BB = 0.0, rz = 0.0, rlast = 0.0, rin = 0.0, RR = 0.0;
+    __shared__ float s_f;   // alpha or beta
+    __shared__ int s_what;  // 0 go on, 1 a reliable update is due, 2 solved
+    if (!cg_sum(sy, bb, [&](double v) { BB = v == 0.0 ? 1.0 : v; }))
         return;
-    double BB = grid_total(part0, s_red);
-    if (BB == 0.0)
-        BB = 1.0;
+
+    // this thread's nodes: their place at the period's ends (bits: i == 0, i == nx - 1),
+    // and the iterates
+    int edge[K > 0 ? K : 1];  // (the plates' p and r are zero: no case of their own)
+    float rk[K > 0 ? K : 1], dk[K > 0 ? K : 1], qk[K > 0 ? K : 1], pk[K > 0 ? K : 1];
+    const int t0 = (int)gtid + first, stride = (int)gstride;
+    auto edge_of = [&](int idx) {
+        const int j = idx / nx, i = idx - j * nx;
+        return (i == 0 ? 1 : 0) | (i == nx - 1 ? 2 : 0);
+    };
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int idx = t0 + k * stride;
+        edge[k] = idx < last ? edge_of(idx) : 0;
+        dk[k] = qk[k] = pk[k] = rk[k] = 0.0f;
+    }
 
     int it = 0;
-    double RR = 0.0;
     // true residual in FP64: r = b - A phi (A phi on the unknowns = the full stencil
     // on phi, plate rows included, plus the plate terms held in b), stored in FP32
     auto true_residual = [&]() -> bool {
         double rr = 0.0;
-        for (long long t = gtid + first; t < last; t += gstride) {
-            const int idx = (int)t;
+        auto one = [&](int idx) {
             const int j = idx / nx, i = idx - j * nx;
             double ap = stencil(p.phi, idx, i, nx);
             if (j == 1)
@@ -1180,91 +1295,151 @@ __global__ void __launch_bounds__(kCgThreads) k_cg2d(Params2D p, int mode)
             if (j == ny - 1)
                 ap += p.phi_hi;
             const double r = __ldcg(b64 + idx) - ap;
-            p.fr[idx] = (float)r;
             rr = fma(r, r, rr);
+            const float f = (float)r;
+            p.fr[idx] = f;
+            return f;
+        };
+        if (K > 0) {
+#pragma unroll
+            for (int k = 0; k < K; ++k)
+                if (t0 + k * stride < last)
+                    rk[k] = one(t0 + k * stride);
+        } else {
+            for (long long t = gtid + first; t < last; t += gstride)
+                one((int)t);
         }
-        rr = block_sum(rr, s_red);
-        if (threadIdx.x == 0)
-            part1[blockIdx.x] = rr;
-        if (!grid_sync(st))
-            return false;
-        RR = grid_total(part1, s_red);
-        return true;
+        return cg_sum(sy, rr, [&](double v) {
+            RR = v;
+            // the FP32 recursion had drifted from the truth (true residual more than twice
+            // the recursive one): its search direction is stale, start afresh
+            const bool restart = it == 0 || RR > 4.0 * rin;
+            const double rz1 = 0.25 * RR;
+            s_f = restart ? 0.0f : cg_quotient(rz1, rz);
+            s_what = RR <= p.rtol2 * BB ? 2 : 0;
+            rz = rz1;
+            rlast = RR;
+        });
     };
     if (!true_residual())
         return;
-    bool done = RR <= p.rtol2 * BB;
-    double rz = 0.25 * RR, beta = 0.0, rin = RR, rlast = RR;
-    bool restart = false;
+    bool done = s_what == 2;
+    float bf = s_f;
     float *pold = p.fpA, *pnew = p.fpB;
     while (!done && it < p.cg_maxit) {
         // phase 1: p = r/4 + beta p_old at the node and its neighbours, q = A p
-        const float bf = (float)beta;
         double pq = 0.0;
-        for (long long t = gtid + first; t < last; t += gstride) {
-            const int idx = (int)t;
-            const int j = idx / nx, i = idx - j * nx;
-            const int ip = (i + 1 == nx) ? idx + 1 - nx : idx + 1;
-            const int im = (i == 0) ? idx - 1 + nx : idx - 1;
-            const float pc = fmaf(bf, __ldcg(pold + idx), 0.25f * __ldcg(p.fr + idx));
-            const float pe = fmaf(bf, __ldcg(pold + ip), 0.25f * __ldcg(p.fr + ip));
-            const float pw = fmaf(bf, __ldcg(pold + im), 0.25f * __ldcg(p.fr + im));
-            const float pn =
-                (j + 1 < ny) ? fmaf(bf, __ldcg(pold + idx + nx), 0.25f * __ldcg(p.fr + idx + nx))
-                             : 0.0f;
-            const float ps =
-                (j > 1) ? fmaf(bf, __ldcg(pold + idx - nx), 0.25f * __ldcg(p.fr + idx - nx)) : 0.0f;
-            const float qv = 4.0f * pc - (pe + pw + pn + ps);
-            pnew[idx] = pc;
-            p.fq[idx] = qv;
-            pq = fma((double)pc, (double)qv, pq);
-        }
-        const double pqs = block_sum(pq, s_red);
-        if (threadIdx.x == 0)
-            part2[blockIdx.x] = pqs;
-        if (!grid_sync(st))
-            return;
-        const double alpha = rz / grid_total(part2, s_red);
-        const float af = (float)alpha;
-        // phase 2: d += alpha p, r -= alpha q
-        double r2 = 0.0;
-        for (long long t = gtid + first; t < last; t += gstride) {
-            const int idx = (int)t;
-            p.fd[idx] = fmaf(af, pnew[idx], p.fd[idx]);
-            const float r = fmaf(-af, p.fq[idx], p.fr[idx]);
-            p.fr[idx] = r;
-            r2 = fma((double)r, (double)r, r2);
-        }
-        const double r2s = block_sum(r2, s_red);
-        if (threadIdx.x == 0)
-            part1[blockIdx.x] = r2s;
-        if (!grid_sync(st))
-            return;
-        rin = grid_total(part1, s_red);
-        ++it;
-        if (rin <= kUpdateDrop * kUpdateDrop * rlast || rin <= 0.25 * p.rtol2 * BB ||
-            it >= p.cg_maxit) {
-            // reliable update: phi += d in FP64, r replaced by the true residual
+        struct Nb {
+            float pe, re, pw, rw, pn, rn, ps, rs;
+        };
+        auto load = [&](int idx, int e) {
+            const int ip = (e & 2) ? idx + 1 - nx : idx + 1;
+            const int im = (e & 1) ? idx - 1 + nx : idx - 1;
+            return Nb{__ldcg(pold + ip),       __ldcg(p.fr + ip),       __ldcg(pold + im),
+                      __ldcg(p.fr + im),       __ldcg(pold + idx + nx), __ldcg(p.fr + idx + nx),
+                      __ldcg(pold + idx - nx), __ldcg(p.fr + idx - nx)};
+        };
+        auto direction = [&](const Nb &n, float po, float ro, float &pc) {
+            pc = fmaf(bf, po, 0.25f * ro);
+            const float pe = fmaf(bf, n.pe, 0.25f * n.re);
+            const float pw = fmaf(bf, n.pw, 0.25f * n.rw);
+            const float pn = fmaf(bf, n.pn, 0.25f * n.rn);
+            const float ps = fmaf(bf, n.ps, 0.25f * n.rs);
+            return 4.0f * pc - (pe + pw + pn + ps);
+        };
+        if (K > 0) {
+            constexpr int kB = K > 0 && K < 4 ? K : 4;  // nodes whose loads are in flight together
+#pragma unroll
+            for (int k0 = 0; k0 < K; k0 += kB) {
+                Nb nb[kB];
+#pragma unroll
+                for (int k = 0; k < kB; ++k)
+                    nb[k] = load(min(t0 + (k0 + k) * stride, last - 1), edge[k0 + k]);
+#pragma unroll
+                for (int k = 0; k < kB; ++k) {
+                    const int idx = t0 + (k0 + k) * stride;
+                    if (idx < last) {
+                        float pc;
+                        const float qv = direction(nb[k], pk[k0 + k], rk[k0 + k], pc);
+                        qk[k0 + k] = qv;
+                        pk[k0 + k] = pc;
+                        pnew[idx] = pc;
+                        pq = fma(cg_double(pc), cg_double(qv), pq);
+                    }
+                }
+            }
+        } else {
             for (long long t = gtid + first; t < last; t += gstride) {
                 const int idx = (int)t;
-                p.phi[idx] += (double)p.fd[idx];
-                p.fd[idx] = 0.0f;
+                float pc;
+                const float qv =
+                    direction(load(idx, edge_of(idx)), __ldcg(pold + idx), __ldcg(p.fr + idx), pc);
+                pnew[idx] = pc;
+                p.fq[idx] = qv;
+                pq = fma(cg_double(pc), cg_double(qv), pq);
             }
-            if (!grid_sync(st))
+        }
+        if (!cg_sum(sy, pq, [&](double v) { s_f = cg_quotient(rz, v); }))  // alpha
+            return;
+        const float af = s_f;
+        // phase 2: d += alpha p, r -= alpha q
+        double r2 = 0.0;
+        if (K > 0) {
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                const int idx = t0 + k * stride;
+                if (idx < last) {
+                    dk[k] = fmaf(af, pk[k], dk[k]);
+                    rk[k] = fmaf(-af, qk[k], rk[k]);
+                    p.fr[idx] = rk[k];
+                    r2 = fma(cg_double(rk[k]), cg_double(rk[k]), r2);
+                }
+            }
+        } else {
+            for (long long t = gtid + first; t < last; t += gstride) {
+                const int idx = (int)t;
+                p.fd[idx] = fmaf(af, pnew[idx], p.fd[idx]);
+                const float r = fmaf(-af, p.fq[idx], p.fr[idx]);
+                p.fr[idx] = r;
+                r2 = fma(cg_double(r), cg_double(r), r2);
+            }
+        }
+        ++it;
+        if (!cg_sum(sy, r2, [&](double v) {
+                rin = v;
+                const bool update = rin <= kUpdateDrop * kUpdateDrop * rlast || rin <= 0.25 * p.rtol2 * BB ||
+                                    it >= p.cg_maxit;
+                s_what = update ? 1 : 0;
+                if (!update) {
+                    const double rz1 = 0.25 * rin;
+                    s_f = cg_quotient(rz1, rz);  // beta
+                    rz = rz1;
+                }
+            }))
+            return;
+        if (s_what == 1) {
+            // reliable update: phi += d in FP64, r replaced by the true residual
+            if (K > 0) {
+#pragma unroll
+                for (int k = 0; k < K; ++k)
+                    if (t0 + k * stride < last) {
+                        p.phi[t0 + k * stride] += (double)dk[k];
+                        dk[k] = 0.0f;
+                    }
+            } else {
+                for (long long t = gtid + first; t < last; t += gstride) {
+                    const int idx = (int)t;
+                    p.phi[idx] += (double)p.fd[idx];
+                    p.fd[idx] = 0.0f;
+                }
+            }
+            if (!cg_sum(sy, 0.0, [](double) {}))
                 return;
             if (!true_residual())
                 return;
-            done = RR <= p.rtol2 * BB;
-            // the FP32 recursion had drifted from the truth (true residual more than
-            // twice the recursive one): its search direction is stale, start afresh
-            restart = RR > 4.0 * rin;
-            rin = RR;
-            rlast = RR;
+            done = s_what == 2;
         }
-        const double rz1 = 0.25 * rin;
-        beta = restart ? 0.0 : rz1 / rz;
-        restart = false;
-        rz = rz1;
+        bf = s_f;
         float *tmp = pold;
         pold = pnew;
         pnew = tmp;
@@ -1280,6 +1455,23 @@ __global__ void __launch_bounds__(kCgThreads) k_cg2d(Params2D p, int mode)
         if (!done)
             atomicCAS(&st->error, 0, SLPIC_ERR_NOCONVERGE);
     }
+}
+
+// the instantiation for a grid: the fewest registers that hold its nodes per thread
+typedef void (*CgKernel)(Params2D, int);
+
+CgKernel cg_kernel(const Params2D &p)
+{
+    const long long threads = (long long)p.cg_v * kCgVirtual, nodes = (long long)(p.ny - 1) * p.nx;
+    const long long k = (nodes + threads - 1) / threads;
+    return k <= 1 ? k_cg2d<1> : k <= 2 ? k_cg2d<2> : k <= 4 ? k_cg2d<4> : k <= 8 ? k_cg2d<8>
+         : k <= 16 ? k_cg2d<16> : k_cg2d<0>;
+}
+
+// CTAs that have nodes
+int cg_grid(const Params2D &p)
+{
+    return (int)std::min<long long>(p.cg_v / 2, ((long long)p.nn + kCgThreads - 1) / kCgThreads);
 }
 
 // ---- the direct solver (SLPIC2D_SOLVER_FFT) -----------------------------------------
@@ -1754,7 +1946,6 @@ struct slpic2d_sim {
     int ctas = 1;     // particle-kernel CTAs per species
     int tile_ctas = 0;  // k_particles2d_tiles CTAs per species (0: not resident)
     int small_ctas = 1; // k_hard2d and k_inject2d: 2 CTAs of 256 threads per SM
-    int cg_ctas = 1;  // cooperative CG grid
     bool prepared = false;
     bool timing = false;               // record events around the kernels of each step
     std::vector<cudaEvent_t> events;   // 4 per recorded step
@@ -1803,7 +1994,8 @@ static int launch_cg(slpic2d_t *h, int mode)
 {
     Params2D p = h->p;
     void *args[] = {&p, &mode};
-    CK2(h, cudaLaunchCooperativeKernel((const void *)k_cg2d, dim3(h->cg_ctas), dim3(kCgThreads),
+    CK2(h, cudaMemsetAsync(p.part, 0xFF, sizeof(double) * 3 * p.cg_v, h->stream));  // kCgEmpty
+    CK2(h, cudaLaunchCooperativeKernel((const void *)cg_kernel(p), dim3(cg_grid(p)), dim3(kCgThreads),
                                        args, 0, h->stream));
     return SLPIC_OK;
 }
@@ -2045,10 +2237,10 @@ extern "C" int slpic2d_create(const slpic2d_config *c, slpic2d_t **out)
     int dev = 0, sms = 1, occ = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_cg2d, kCgThreads, 0) != cudaSuccess ||
+    p.cg_v = std::min(2 * sms, kCgMaxVirtual);
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, cg_kernel(p), kCgThreads, 0) != cudaSuccess ||
         occ < 1)
         return bail(SLPIC_ERR_CUDA, "CG kernel occupancy query failed");
-    h->cg_ctas = std::min(sms * std::min(occ, 2), kBarGroup * kBarGroups);
     h->ctas = sms * 4;
     h->small_ctas = sms * 2;
     {
@@ -2062,7 +2254,7 @@ extern "C" int slpic2d_create(const slpic2d_config *c, slpic2d_t **out)
             h->tile_ctas = std::max(1, sms * occ_t / p.ns);
         cudaGetLastError();
     }
-    if (!alloc((void **)&p.part, sizeof(double) * 3 * h->cg_ctas))
+    if (!alloc((void **)&p.part, sizeof(double) * 3 * p.cg_v))
         return bail(SLPIC_ERR_OOM, "device allocation failed");
     if (!alloc((void **)&p.hist, sizeof(int) * nn) || !alloc((void **)&p.cursor, sizeof(int) * nn) ||
         !alloc((void **)&p.bsum, sizeof(int) * ((nn + kScanBlock - 1) / kScanBlock + 1)))
