@@ -201,7 +201,9 @@ int slpic_prepare(slpic_t *h);
  * beta(|v^{n+1/2}|) v^{n+1/2} dt, absorb at walls (or wrap), deposit
  * rho^{n+1}; then inject source particles (deposited into rho^{n+1}, first
  * pushed next step) and solve phi^{n+1}, E^{n+1}.  The steps run as a
- * captured CUDA graph with no host synchronisation between them. */
+ * captured CUDA graph with no host synchronisation between them; a call of 4 or
+ * more steps of a simulation of at most 15 million slots (capacities) runs them
+ * in one launch instead (at most 4096 steps each), with the same results. */
 int slpic_step(slpic_t *h, int64_t nsteps);
 
 /* Wait for queued work; report device-side errors raised since the last
@@ -295,7 +297,10 @@ int slpic_set_wait_limit(slpic_t *h, int64_t cycles);
  * iterative push) and 2 (the source and field kernel), ms[kind] is the summed
  * device time of its launches since the handle was created, each launch counted
  * from the start of its first CTA to the end of its last on the GPU's global timer,
- * and launches[kind] the number of launches.  Differences of two calls give the
+ * and launches[kind] the number of launches.  Where many steps run in one launch, each
+ * step counts as one of every kind, with the times of the first CTA's phases: its
+ * particles; the iterative pushes and the hand-over of its charge; the wait for the other
+ * CTAs, the source and the field.  Differences of two calls give the
  * time of the steps between them.  Synchronising; either pointer may be NULL;
  * SLPIC_ERR_INVALID for a batch handle. */
 int slpic_kernel_spans(slpic_t *h, double *ms, int64_t *launches);

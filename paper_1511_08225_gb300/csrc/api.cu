@@ -2,7 +2,8 @@
 //
 // The handle owns all device memory of one simulation; the timestep runs as a
 // captured CUDA graph (particle kernel, then field kernel) whose kernels read
-// the time level from device memory, so one graph serves every step.
+// the time level from device memory, so one graph serves every step, or, for
+// simulations that are not large, as many steps in one launch (k_steps).
 #include <cmath>
 #include <cstdio>
 #include <algorithm>
@@ -31,6 +32,8 @@ struct slpic_sim {
     int ctas_c = 1;      // compacting particle-kernel CTAs per species
     int hard_ctas = 1;   // k_hard CTAs
     int tma_stages = 0;  // k_particles_tma ring stages for in-place steps (0: k_particles)
+    void *d_steps = nullptr;  // scratch of k_steps (null: the simulation is not small)
+    int steps_ctas = 0, steps_smem = 0;  // its CTAs; the shared memory it may take
     // performance settings (slpic_set_tuning / slpic_autotune); results do not depend
     // on them
     int compact_every = kCompactEvery;  // a compacting particle step every this many
@@ -257,6 +260,7 @@ static void free_all(slpic_t *h)
     cudaFree(h->d_bad);
     cudaFree(h->d_lam);
     cudaFree(h->d_stage);
+    cudaFree(h->d_steps);
     for (int s = 0; s < kMaxSpecies; ++s) {
         for (int b = 0; b < 2; ++b) {
             cudaFree(h->d_cell[s][b]);
@@ -377,6 +381,22 @@ extern "C" int slpic_create(const slpic_config *cfg, slpic_t **out)
     // per SM, whose idle CTAs cost about a microsecond
     h->hard_ctas = sms * 2;
     CKC(configure_particles_tma(nn, &h->tma_stages));
+    // small simulations: many steps in one launch (k_steps)
+    {
+        long long slots = 0, most = 0;
+        for (int s = 0; s < ns; ++s) {
+            slots += cfg->species[s].capacity;
+            most = std::max(most, (long long)cfg->species[s].capacity);
+        }
+        CKC(configure_steps(&h->steps_smem));
+        if (slots <= kStepsMaxSlots && most <= kStepsMaxSpecies &&
+            steps_smem_bytes(nn, ns, true) <= (size_t)h->steps_smem) {
+            CKC(cudaMalloc(&h->d_steps, steps_scratch_bytes(nn, ns)));
+            // a CTA per SM (one SM left free, as for the TMA kernel), fewer where that
+            // would leave each less than a warp's worth of every scheduler
+            h->steps_ctas = (int)std::max(1LL, std::min((long long)sms - 1, (slots + 767) / 768));
+        }
+    }
 
     StepParams &p = h->p;
     p.n_cells = cfg->n_cells;
@@ -666,6 +686,15 @@ static int capture(slpic_t *h, long long first_step, int nsteps, bool timed,
     return SLPIC_OK;
 }
 
+// Whether a call of nsteps steps runs in one launch (k_steps): a small simulation and more
+// than a few steps, none of the modes that k_steps does not have (the prescribed wave,
+// timed graphs, the per-warp kernel, a changed wait limit, which is the TMA kernel's).
+static bool steps_fused(const slpic_t *h, int64_t nsteps)
+{
+    return h->d_steps && nsteps >= kStepsFewest && !h->p.wave_on && h->t_len == 0 && h->particle_kernel == 0 &&
+           h->p.wait_cycles == kWaitCycles;
+}
+
 extern "C" int slpic_step(slpic_t *h, int64_t nsteps)
 {
     int rc = check_handle(h, 0);
@@ -679,6 +708,15 @@ extern "C" int slpic_step(slpic_t *h, int64_t nsteps)
         return rc;
     if (nsteps == 0)
         return SLPIC_OK;
+    if (steps_fused(h, nsteps)) {
+        for (int64_t left = nsteps; left > 0;) {
+            const int n = (int)std::min<int64_t>(left, kStepsMost);
+            CK(h, launch_steps(h->p, n, h->compact_every, h->steps_ctas, h->d_steps, h->stream));
+            h->step += n;
+            left -= n;
+        }
+        return SLPIC_OK;
+    }
     // graphs: steps whose index is 0 mod compact_every start a cycle
     if (!h->g1 && (rc = capture(h, 0, 1, false, &h->g1)))
         return rc;

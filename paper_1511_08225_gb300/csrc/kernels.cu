@@ -46,13 +46,6 @@ namespace slpic {
 // from that start to its own end.  A few atomics per CTA; the next launch of the
 // same kernel follows on the stream, so the reset cannot race it.
 // ---------------------------------------------------------------------------------
-__device__ __forceinline__ unsigned long long gtimer()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
-}
-
 __device__ __forceinline__ void span_enter(DevState *st, int k)
 {
     if (threadIdx.x == 0)
@@ -959,68 +952,24 @@ __device__ double block_sum(double v, double *s_w)
     return t;
 }
 
-// Source particle i of species s for this step (Sec. IV source, the readings of
-// LOSS_MATCHED / RATE): it takes uniforms u_j = u24(SplitMix64(key, 8i+j)), key the
-// species' stream of the step, for its position in the band (FP32, pinned
-// operations) and a physical Maxwellian velocity (Box-Muller): the g-source equals
-// the f-source.  It goes to slot base + i of buffer Q, its deposit to acc[Q].
+// Source particle i of species s goes to slot base + i of buffer Q, its deposit to acc[Q].
 __device__ __forceinline__ void inject_one(const StepParams &p, int s, unsigned long long key,
                                            long long base, long long i, int Q)
 {
     const SpeciesDev &sp = p.sp[s];
-    const int N = p.n_cells;
     unsigned long long *acc = p.acc + ((size_t)Q * p.ns + s) * p.nn;
-    {
-        unsigned long long b8 = 8ULL * (unsigned long long)i;
-        float u0 = u24(sm64_at(key, b8 + 0));
-        float u1 = u24(sm64_at(key, b8 + 1));
-        float u2 = u24(sm64_at(key, b8 + 2));
-        float u3 = u24(sm64_at(key, b8 + 3));
-        float u4 = u24(sm64_at(key, b8 + 4));
-        int c;
-        float off;
-        float4 q;
-        if (p.src_mode == SLPIC_SRC_WALL) {
-            // through the plate at x = L: the flux-weighted half-Maxwellian (|vx|
-            // Rayleigh, towards -x), placed where it has moved since a uniformly
-            // random entry time in the step; a position that rounds to the plate is
-            // put at the largest cell coordinate below it
-            const float vxm = sp.vth_src * sqrtf(-2.0f * logf(u1));
-            const float rw = sp.vth_src * sqrtf(-2.0f * logf(u2));
-            float sw, cw;
-            sincospif(2.0f * u3, &sw, &cw);
-            const float vy = rw * cw, vz = rw * sw;
-            const float b = beta_q(sp.kind, -vxm, vy, vz, v0_cell(p, sp, N - 1));
-            float xc = __fsub_rn((float)N, __fmul_rn(u0, __fmul_rn(__fmul_rn(b, vxm), p.dt_dx)));
-            if (!(xc < (float)N))
-                xc = __int_as_float(__float_as_int((float)N) - 1);
-            xc = fmaxf(xc, 0.0f);
-            const float fc = floorf(xc);
-            c = (int)fc;
-            off = xc - fc;
-            q = make_float4(off, -vxm, vy, vz);
-        } else {
-            float xc = __fadd_rn(p.src_lo_cells, __fmul_rn(u0, p.src_len_cells));
-            float fc = floorf(xc);
-            c = (int)fc;
-            off = xc - fc;
-            // physical Maxwellian (Box-Muller); the g-source equals the f-source
-            float r1 = sqrtf(-2.0f * logf(u1)), r2 = sqrtf(-2.0f * logf(u3));
-            float s2, c2;
-            sincospif(2.0f * u2, &s2, &c2);
-            q = make_float4(off, sp.vth_src * r1 * c2, sp.vth_src * r1 * s2,
-                            sp.vth_src * r2 * cospif(2.0f * u4));
-        }
-        sp.cell[Q][base + i] = c;
-        sp.pv[Q][base + i] = q;
-        int c1 = c + 1;
-        if (p.periodic && c1 == N)
-            c1 = 0;
-        unsigned long long qL, qR;
-        quantise(beta_q(sp.kind, q.y, q.z, q.w, v0_cell(p, sp, c)), off, qL, qR);
-        atomicAdd(acc + c, qL);
-        atomicAdd(acc + c1, qR);
-    }
+    int c;
+    float4 q;
+    source_particle(p, sp, key, i, c, q);
+    sp.cell[Q][base + i] = c;
+    sp.pv[Q][base + i] = q;
+    int c1 = c + 1;
+    if (p.periodic && c1 == p.n_cells)
+        c1 = 0;
+    unsigned long long qL, qR;
+    quantise(beta_q(sp.kind, q.y, q.z, q.w, v0_cell(p, sp, c)), q.x, qL, qR);
+    atomicAdd(acc + c, qL);
+    atomicAdd(acc + c1, qR);
 }
 
 // The step's source particles of every species (k[s] of species s, to slots base[s]
@@ -1286,25 +1235,8 @@ __device__ __forceinline__ void field_body(const StepParams &p, int mode)
         // exchange below, when every CTA has read the state.
         const int s = threadIdx.x;
         if (s < ns) {
-            double S = 0.0;
-            if (p.src_mode == SLPIC_SRC_LOSS_MATCHED) {
-                S = (double)(pf_ref0 + pf_ref1) * p.sp[p.src_ref].w;
-            } else if (p.src_mode == SLPIC_SRC_RATE) {
-                S = p.src_rate * p.dt64;
-            }
-            long long k = 0;
             double f = pf_frac;
-            if (p.src_mode == SLPIC_SRC_WALL) {
-                if (p.sp[s].wall_rate > 0.0) {
-                    f += p.sp[s].wall_rate;
-                    k = (long long)floor(f);
-                    f -= (double)k;
-                }
-            } else if (p.src_mode != SLPIC_SRC_NONE && p.sp[s].vth_src > 0.0f) {
-                f = fma(S, p.sp[s].inv_w, f);
-                k = (long long)floor(f);
-                f -= (double)k;
-            }
+            const long long k = source_count(p, p.sp[s], pf_ref0 + pf_ref1, f);
             // after an in-place step the output uses the input's slots (holes
             // included); after a compacting step its count was reserved by atomics
             long long have = (long long)(mode == 1 ? (P ? pf_cnt1 : pf_cnt0) : (P ? pf_cnt0 : pf_cnt1));

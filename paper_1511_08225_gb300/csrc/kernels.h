@@ -37,6 +37,19 @@ size_t particle_tma_smem_bytes(int nn, int stages);
 // ring stages that fit beside an nn-node grid (at most 4); 0 if fewer than 2 fit
 cudaError_t configure_particles_tma(int nn, int *stages);
 void launch_particles_tma(const StepParams &p, int ctas, int stages, cudaStream_t st);
+// k_steps (steps.cu): many steps in one cooperative launch of `ctas` CTAs; scratch of
+// steps_scratch_bytes on the device; max_smem: dynamic shared memory it may take
+constexpr int kStepsThreads = 1024;
+// Where the line lies (us a step, three kernels against k_steps): 2,560 particles 27 / 9,
+// 51,200 30 / 12, 5.2e5 42 / 25, 2.0e6 62 / 47, 4.9e6 83 / 75 (14.7M slots), 8.2e6 112 /
+// 114.  The host knows the slots, of which a third to all are in use.
+constexpr long long kStepsMaxSlots = 15000000;        // most slots, all species
+constexpr long long kStepsMaxSpecies = (1LL << 24) - 1;  // ... and of one: its sums fit 64 bits
+constexpr int kStepsFewest = 4, kStepsMost = 4096;  // steps of a launch
+size_t steps_scratch_bytes(int nn, int ns);
+size_t steps_smem_bytes(int nn, int ns, bool profile);
+cudaError_t configure_steps(int *max_smem);
+cudaError_t launch_steps(const StepParams &p, int nsteps, int every, int ctas, void *scratch, cudaStream_t st);
 void launch_hard(const StepParams &p, int ctas, bool compact, cudaStream_t st);
 void launch_field(const StepParams &p, int mode, cudaStream_t st);
 // copy of a deposit ([species][nn], ndep words) and of E, for an overlapped read-back

@@ -144,4 +144,81 @@ __device__ __forceinline__ bool advance(const StepParams &p, const SpeciesDev &s
     return move_and_deposit(p, sp, dep, c, q, vx, wall, sp.v0);
 }
 
+// Source particle i of species s for the step (Sec. IV source, the readings of
+// LOSS_MATCHED / RATE): it takes uniforms u_j = u24(SplitMix64(key, 8i+j)), key the
+// species' stream of the step, for its position in the band (FP32, pinned
+// operations) and a physical Maxwellian velocity (Box-Muller): the g-source equals
+// the f-source.
+__device__ __forceinline__ void source_particle(const StepParams &p, const SpeciesDev &sp,
+                                                unsigned long long key, long long i, int &c, float4 &q)
+{
+    const int N = p.n_cells;
+    const unsigned long long b8 = 8ULL * (unsigned long long)i;
+    const float u0 = u24(sm64_at(key, b8 + 0)), u1 = u24(sm64_at(key, b8 + 1));
+    const float u2 = u24(sm64_at(key, b8 + 2)), u3 = u24(sm64_at(key, b8 + 3));
+    const float u4 = u24(sm64_at(key, b8 + 4));
+    if (p.src_mode == SLPIC_SRC_WALL) {
+        // through the plate at x = L: the flux-weighted half-Maxwellian (|vx|
+        // Rayleigh, towards -x), placed where it has moved since a uniformly
+        // random entry time in the step; a position that rounds to the plate is
+        // put at the largest cell coordinate below it
+        const float vxm = sp.vth_src * sqrtf(-2.0f * logf(u1));
+        const float rw = sp.vth_src * sqrtf(-2.0f * logf(u2));
+        float sw, cw;
+        sincospif(2.0f * u3, &sw, &cw);
+        const float vy = rw * cw, vz = rw * sw;
+        const float b = beta_q(sp.kind, -vxm, vy, vz, v0_cell(p, sp, N - 1));
+        float xc = __fsub_rn((float)N, __fmul_rn(u0, __fmul_rn(__fmul_rn(b, vxm), p.dt_dx)));
+        if (!(xc < (float)N))
+            xc = __int_as_float(__float_as_int((float)N) - 1);
+        xc = fmaxf(xc, 0.0f);
+        const float fc = floorf(xc);
+        c = (int)fc;
+        q = make_float4(xc - fc, -vxm, vy, vz);
+    } else {
+        const float xc = __fadd_rn(p.src_lo_cells, __fmul_rn(u0, p.src_len_cells));
+        const float fc = floorf(xc);
+        c = (int)fc;
+        // physical Maxwellian (Box-Muller); the g-source equals the f-source
+        const float r1 = sqrtf(-2.0f * logf(u1)), r2 = sqrtf(-2.0f * logf(u3));
+        float s2, c2;
+        sincospif(2.0f * u2, &s2, &c2);
+        q = make_float4(xc - fc, sp.vth_src * r1 * c2, sp.vth_src * r1 * s2,
+                        sp.vth_src * r2 * cospif(2.0f * u4));
+    }
+}
+
+// The step's source count of a species: macroparticles k to make, given the ref species'
+// absorbed macroparticles of the step and the fraction carried (updated).
+__device__ __forceinline__ long long source_count(const StepParams &p, const SpeciesDev &sp,
+                                                  unsigned long long ref_absorbed, double &frac)
+{
+    double S = 0.0;
+    if (p.src_mode == SLPIC_SRC_LOSS_MATCHED)
+        S = (double)ref_absorbed * p.sp[p.src_ref].w;
+    else if (p.src_mode == SLPIC_SRC_RATE)
+        S = p.src_rate * p.dt64;
+    long long k = 0;
+    if (p.src_mode == SLPIC_SRC_WALL) {
+        if (sp.wall_rate > 0.0) {
+            frac += sp.wall_rate;
+            k = (long long)floor(frac);
+            frac -= (double)k;
+        }
+    } else if (p.src_mode != SLPIC_SRC_NONE && sp.vth_src > 0.0f) {
+        frac = fma(S, sp.inv_w, frac);
+        k = (long long)floor(frac);
+        frac -= (double)k;
+    }
+    return k;
+}
+
+// the GPU's global timer, ns
+__device__ __forceinline__ unsigned long long gtimer()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
 }  // namespace slpic
