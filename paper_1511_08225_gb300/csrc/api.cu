@@ -79,6 +79,12 @@ struct slpic_sim {
     float *d_snap_E = nullptr;
     bool rb_used = false;
 
+    // page-locked staging of the synchronising read-backs, so that their copies are queued
+    // behind one another and waited for once (a member of a batch uses the batch's)
+    char *h_stage = nullptr;
+    size_t h_stage_bytes = 0;
+    slpic_sim *batch = nullptr;
+
     std::vector<slpic_sim *> members;
     StepParams *d_params = nullptr;  // [members] on the device
     int4 *d_work = nullptr;          // particle-kernel work items
@@ -261,6 +267,7 @@ static void free_all(slpic_t *h)
     cudaFree(h->d_lam);
     cudaFree(h->d_stage);
     cudaFree(h->d_steps);
+    cudaFreeHost(h->h_stage);
     for (int s = 0; s < kMaxSpecies; ++s) {
         for (int b = 0; b < 2; ++b) {
             cudaFree(h->d_cell[s][b]);
@@ -752,6 +759,45 @@ extern "C" int slpic_step(slpic_t *h, int64_t nsteps)
     return SLPIC_OK;
 }
 
+// Page-locked staging for `bytes` after its first kStageHead, where wait_status puts the
+// device's error; kept for the next read-back.
+constexpr size_t kStageHead = 64;
+
+static int host_stage(slpic_t *h, size_t bytes, char **out)
+{
+    slpic_t *o = h->batch ? h->batch : h;
+    if (bytes + kStageHead > o->h_stage_bytes) {
+        cudaFreeHost(o->h_stage);
+        o->h_stage = nullptr;
+        o->h_stage_bytes = 0;
+        const size_t n = (bytes + kStageHead + 65535) & ~size_t(65535);
+        CK(h, cudaMallocHost((void **)&o->h_stage, n));
+        o->h_stage_bytes = n;
+    }
+    *out = o->h_stage;
+    return SLPIC_OK;
+}
+
+// Wait for everything queued, the caller's copies into the staging among it; the device's
+// error, if one was raised since the last report.
+static int wait_status(slpic_t *h, char *stage)
+{
+    CK(h, cudaMemcpyAsync(stage, &h->d_state->error, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    CK(h, cudaStreamSynchronize(h->stream));
+    if (h->rb_stream)
+        CK(h, cudaStreamSynchronize(h->rb_stream));
+    int e;
+    std::memcpy(&e, stage, sizeof(e));
+    if (e) {
+        int zero = 0;
+        CK(h, cudaMemcpy(&h->d_state->error, &zero, sizeof(int), cudaMemcpyHostToDevice));
+        return fail(h, e, e == SLPIC_ERR_CAPACITY  ? "particle store full: injection truncated"
+                          : e == SLPIC_ERR_TIMEOUT ? "a bounded wait of a particle or step kernel ran out"
+                                                   : "device error");
+    }
+    return SLPIC_OK;
+}
+
 extern "C" int slpic_synchronize(slpic_t *h)
 {
     int rc = check_handle(h, 0);
@@ -766,19 +812,10 @@ extern "C" int slpic_synchronize(slpic_t *h)
             }
         return SLPIC_OK;
     }
-    CK(h, cudaStreamSynchronize(h->stream));
-    if (h->rb_stream)
-        CK(h, cudaStreamSynchronize(h->rb_stream));
-    int e = 0;
-    CK(h, cudaMemcpy(&e, &h->d_state->error, sizeof(int), cudaMemcpyDeviceToHost));
-    if (e) {
-        int zero = 0;
-        CK(h, cudaMemcpy(&h->d_state->error, &zero, sizeof(int), cudaMemcpyHostToDevice));
-        return fail(h, e, e == SLPIC_ERR_CAPACITY  ? "particle store full: injection truncated"
-                          : e == SLPIC_ERR_TIMEOUT ? "a bounded wait of the particle kernel ran out"
-                                                   : "device error");
-    }
-    return SLPIC_OK;
+    char *stage;
+    if ((rc = host_stage(h, 0, &stage)))
+        return rc;
+    return wait_status(h, stage);
 }
 
 static int sync_prepared(slpic_t *h, int instance)
@@ -794,22 +831,38 @@ static int sync_prepared(slpic_t *h, int instance)
 extern "C" int slpic_fields(slpic_t *h, int instance, double *rho, double *phi, float *E)
 {
     BATCH_FORWARD(h, instance, slpic_fields(m_, 0, rho, phi, E));
-    int rc = sync_prepared(h, instance);
+    int rc = check_handle(h, instance);
     if (rc)
         return rc;
+    if (h->dirty && (rc = slpic_prepare(h)))
+        return rc;
+    const size_t b8 = sizeof(double) * h->nn, b4 = sizeof(float) * h->nn;
+    char *stage;
+    if ((rc = host_stage(h, 2 * b8 + b4, &stage)))
+        return rc;
+    char *s_rho = stage + kStageHead, *s_phi = s_rho + b8, *s_E = s_phi + b8;
     if (rho || phi) {
         // the step computes E only; rho and phi of the latest deposit on demand
+        if (h->rb_used)  // an overlapped read-back may still be copying them
+            CK(h, cudaStreamWaitEvent(h->stream, h->ev_rb, 0));
         launch_potential(h->p, h->d_acc + (size_t)(h->step & 1) * h->ns * h->nn, h->step,
                          h->stream);
         CK(h, cudaGetLastError());
-        CK(h, cudaStreamSynchronize(h->stream));
     }
     if (rho)
-        CK(h, cudaMemcpy(rho, h->d_rho, sizeof(double) * h->nn, cudaMemcpyDeviceToHost));
+        CK(h, cudaMemcpyAsync(s_rho, h->d_rho, b8, cudaMemcpyDeviceToHost, h->stream));
     if (phi)
-        CK(h, cudaMemcpy(phi, h->d_phi, sizeof(double) * h->nn, cudaMemcpyDeviceToHost));
+        CK(h, cudaMemcpyAsync(s_phi, h->d_phi, b8, cudaMemcpyDeviceToHost, h->stream));
     if (E)
-        CK(h, cudaMemcpy(E, h->d_E, sizeof(float) * h->nn, cudaMemcpyDeviceToHost));
+        CK(h, cudaMemcpyAsync(s_E, h->d_E, b4, cudaMemcpyDeviceToHost, h->stream));
+    if ((rc = wait_status(h, stage)))
+        return rc;
+    if (rho)
+        std::memcpy(rho, s_rho, b8);
+    if (phi)
+        std::memcpy(phi, s_phi, b8);
+    if (E)
+        std::memcpy(E, s_E, b4);
     return SLPIC_OK;
 }
 
@@ -857,14 +910,25 @@ extern "C" int slpic_fields_async(slpic_t *h, int instance, double *rho, double 
 extern "C" int slpic_charge_raw(slpic_t *h, int instance, int species, int64_t *acc)
 {
     BATCH_FORWARD(h, instance, slpic_charge_raw(m_, 0, species, acc));
-    int rc = sync_prepared(h, instance);
+    int rc = check_handle(h, instance);
     if (rc)
         return rc;
-    if (species < 0 || species >= h->ns || !acc)
+    if (h->dirty && (rc = slpic_prepare(h)))
+        return rc;
+    const bool valid = species >= 0 && species < h->ns && acc;
+    const size_t b = sizeof(int64_t) * h->nn;
+    char *stage;
+    if ((rc = host_stage(h, b, &stage)))
+        return rc;
+    if (valid)
+        CK(h, cudaMemcpyAsync(stage + kStageHead,
+                              h->d_acc + ((size_t)(h->step & 1) * h->ns + species) * h->nn, b,
+                              cudaMemcpyDeviceToHost, h->stream));
+    if ((rc = wait_status(h, stage)))
+        return rc;
+    if (!valid)
         return fail(h, SLPIC_ERR_INVALID, "bad species or pointer");
-    const int P = (int)(h->step & 1);
-    CK(h, cudaMemcpy(acc, h->d_acc + ((size_t)P * h->ns + species) * h->nn,
-                     sizeof(int64_t) * h->nn, cudaMemcpyDeviceToHost));
+    std::memcpy(acc, stage + kStageHead, b);
     return SLPIC_OK;
 }
 
@@ -1404,8 +1468,10 @@ extern "C" int slpic_create_batch(const slpic_config *cfgs, int m, slpic_t **out
         cudaStreamCreateWithFlags(&h->cap_stream, cudaStreamNonBlocking) != cudaSuccess)
         return bail(SLPIC_ERR_CUDA, "stream creation failed");
     h->stream = h->own_stream;
-    for (slpic_t *x : members)
+    for (slpic_t *x : members) {
         x->stream = h->stream;
+        x->batch = h;
+    }
     if (cudaMalloc(&h->d_params, sizeof(StepParams) * m) != cudaSuccess)
         return bail(SLPIC_ERR_OOM, "device allocation failed");
     int occ = 0, occ_c = 0;

@@ -23,6 +23,7 @@
 // cells: the particle kernel 819 us a step, now 46).
 #include <algorithm>
 #include <cmath>
+#include <cstring>
 #include <string>
 #include <vector>
 
@@ -655,6 +656,7 @@ struct slpic_fp64_sim {
     cudaStream_t stream = nullptr, own_stream = nullptr;
     P64 p{};
     int ctas = 1;
+    char *h_stage = nullptr;  // page-locked: the state, then rho, phi and E, for slpic_fp64_fields
     std::vector<void *> allocs;
     std::string err;
 };
@@ -784,6 +786,7 @@ extern "C" int slpic_fp64_destroy(slpic_fp64_t *h)
         cudaStreamSynchronize(h->own_stream);
     for (void *a : h->allocs)
         cudaFree(a);
+    cudaFreeHost(h->h_stage);
     if (h->own_stream)
         cudaStreamDestroy(h->own_stream);
     delete h;
@@ -884,16 +887,22 @@ extern "C" int slpic_fp64_fields(slpic_fp64_t *h, double *rho, double *phi, doub
 {
     if (!h)
         return SLPIC_ERR_INVALID;
-    int rc = slpic_fp64_synchronize(h);
-    if (rc)
-        return rc;
-    const size_t b = sizeof(double) * h->p.nn;
-    if (rho)
-        CK64(h, cudaMemcpy(rho, h->p.rho, b, cudaMemcpyDeviceToHost));
-    if (phi)
-        CK64(h, cudaMemcpy(phi, h->p.phi, b, cudaMemcpyDeviceToHost));
-    if (E)
-        CK64(h, cudaMemcpy(E, h->p.E, b, cudaMemcpyDeviceToHost));
+    // the state's error and the fields queued into page-locked memory, one wait
+    const size_t b = sizeof(double) * h->p.nn, head = (sizeof(St64) + 63) & ~size_t(63);
+    if (!h->h_stage)
+        CK64(h, cudaMallocHost((void **)&h->h_stage, head + 3 * b));
+    CK64(h, cudaMemcpyAsync(h->h_stage, h->p.st, sizeof(St64), cudaMemcpyDeviceToHost, h->stream));
+    const double *src[3] = {h->p.rho, h->p.phi, h->p.E};
+    double *dst[3] = {rho, phi, E};
+    for (int k = 0; k < 3; ++k)
+        if (dst[k])
+            CK64(h, cudaMemcpyAsync(h->h_stage + head + k * b, src[k], b, cudaMemcpyDeviceToHost, h->stream));
+    CK64(h, cudaStreamSynchronize(h->stream));
+    if (reinterpret_cast<const St64 *>(h->h_stage)->error)
+        return slpic_fp64_synchronize(h);
+    for (int k = 0; k < 3; ++k)
+        if (dst[k])
+            std::memcpy(dst[k], h->h_stage + head + k * b, b);
     return SLPIC_OK;
 }
 

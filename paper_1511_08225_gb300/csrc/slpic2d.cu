@@ -1880,6 +1880,32 @@ __global__ void __launch_bounds__(kThreads) k_sort_scatter2d(Params2D p, int s, 
     }
 }
 
+// ---- read-back (slpic2d_fields): rho from the deposits, which are cleared, with the
+// operations of the solves; E's components apart
+__global__ void __launch_bounds__(kThreads) k_rho2d(Params2D p, double *__restrict__ out)
+{
+    for (long long t = (long long)blockIdx.x * kThreads + threadIdx.x; t < p.nn;
+         t += (long long)gridDim.x * kThreads) {
+        double v = 0.0;
+        for (int s = 0; s < p.ns; ++s) {
+            unsigned long long *a = p.acc + (size_t)s * p.nn + t;
+            v = fma(p.sp[s].rho_unit, (double)(long long)*a, v);
+            *a = 0ULL;
+        }
+        out[t] = v;
+    }
+}
+
+__global__ void __launch_bounds__(kThreads) k_split2d(Params2D p, float *__restrict__ ex, float *__restrict__ ey)
+{
+    for (long long t = (long long)blockIdx.x * kThreads + threadIdx.x; t < p.nn;
+         t += (long long)gridDim.x * kThreads) {
+        const float2 e = p.E[t];
+        ex[t] = e.x;
+        ey[t] = e.y;
+    }
+}
+
 // ---- initial guess of the CG (slpic2d_set_warm_start) ------------------------------
 // rho of rows 0..ny-1 as FP32 from the deposits (left in place for the CG kernel);
 // row 0, a plate, is zero.  The layout is the nodal one, so the array is the
@@ -2544,35 +2570,29 @@ extern "C" int slpic2d_fields(slpic2d_t *h, double *rho, double *phi, float *Ex,
         return rc;
     const Params2D &p = h->p;
     const size_t nn = (size_t)p.nn;
+    const unsigned grid = (unsigned)std::min<size_t>((nn + kThreads - 1) / kThreads, 152 * 8);
     if (phi)
-        CK2(h, cudaMemcpy(phi, p.phi, sizeof(double) * nn, cudaMemcpyDeviceToHost));
+        CK2(h, cudaMemcpyAsync(phi, p.phi, sizeof(double) * nn, cudaMemcpyDeviceToHost, h->stream));
     if (Ex || Ey) {
-        std::vector<float2> e(nn);
-        CK2(h, cudaMemcpy(e.data(), p.E, sizeof(float2) * nn, cudaMemcpyDeviceToHost));
-        for (size_t k = 0; k < nn; ++k) {
-            if (Ex)
-                Ex[k] = e[k].x;
-            if (Ey)
-                Ey[k] = e[k].y;
-        }
+        // the components apart, in two of the CG's vectors (free between solves)
+        k_split2d<<<grid, kThreads, 0, h->stream>>>(p, p.fr, p.fq);
+        CK2(h, cudaGetLastError());
+        if (Ex)
+            CK2(h, cudaMemcpyAsync(Ex, p.fr, sizeof(float) * nn, cudaMemcpyDeviceToHost, h->stream));
+        if (Ey)
+            CK2(h, cudaMemcpyAsync(Ey, p.fq, sizeof(float) * nn, cudaMemcpyDeviceToHost, h->stream));
     }
     if (rho) {
-        // rho of the current level from the deposits of the particles now stored
-        // (the consumed deposit was cleared by the solve): recomputed here
+        // rho of the current level from the deposits of the particles now stored (the consumed
+        // deposit was cleared by the solve): made again here, in the vector of a standalone
+        // solve's charge, and the deposits cleared
         CK2(h, cudaMemsetAsync(p.acc, 0, sizeof(unsigned long long) * nn * p.ns, h->stream));
         k_deposit2d<<<dim3(h->ctas, p.ns), kThreads, 0, h->stream>>>(p);
+        k_rho2d<<<grid, kThreads, 0, h->stream>>>(p, p.r);
         CK2(h, cudaGetLastError());
-        CK2(h, cudaStreamSynchronize(h->stream));
-        std::vector<long long> a(nn * p.ns);
-        CK2(h, cudaMemcpy(a.data(), p.acc, sizeof(long long) * nn * p.ns, cudaMemcpyDeviceToHost));
-        CK2(h, cudaMemsetAsync(p.acc, 0, sizeof(unsigned long long) * nn * p.ns, h->stream));
-        for (size_t k = 0; k < nn; ++k) {
-            double v = 0.0;
-            for (int s = 0; s < p.ns; ++s)
-                v = std::fma(p.sp[s].rho_unit, (double)a[(size_t)s * nn + k], v);
-            rho[k] = v;
-        }
+        CK2(h, cudaMemcpyAsync(rho, p.r, sizeof(double) * nn, cudaMemcpyDeviceToHost, h->stream));
     }
+    CK2(h, cudaStreamSynchronize(h->stream));
     return SLPIC_OK;
 }
 
