@@ -54,21 +54,11 @@ constexpr int kCgMaxVirtual = 512;             // virtual CTAs (two per SM)
 constexpr long long kCgWaitCycles = 2000000000LL;  // bounded wait for the other CTAs (~1 s)
 constexpr long long kMaxTimedSteps2d = 4096;    // steps recorded by the kernel timing
 
-// A particle whose push needs the piece walk, listed by the in-place tile kernel
-// for k_hard2d with what the push needs.
-struct HardRec2D {
-    int32_t slot, cell;  // its slot in the step's buffers; c at time level n
-    float ax, ay;        // (q/m) E gathered at the particle
-    float4 q;            // {ox, oy, vx, vy} at time level n (v = v^{n-1/2})
-    float vz, pad[3];
-};
-
 struct Species2D {
     int32_t *cell[2];
     float4 *pv[2];
     float *vz[2];
-    HardRec2D *hard;     // this step's listed particles (hard_cap records)
-    long long hard_cap;
+    int32_t *hard;       // slots of this step's particles whose push needs the walk [capacity]
     long long capacity;
     float qm, v0, vth_src;
     int kind;
@@ -201,6 +191,19 @@ __device__ __forceinline__ bool push_v2_easy(int kind, float ux, float uy, float
     return push_v2_impl<true>(kind, ux, uy, uz, ax, ay, dt, v0, vx, vy);
 }
 
+// (q/m) E at a particle from its cell's four nodes, bilinear, in a fixed operation order
+__device__ __forceinline__ void accel2d(float qm, float2 e00, float2 e10, float2 e01, float2 e11,
+                                        float ox, float oy, float &ax, float &ay)
+{
+    const float wx0 = __fsub_rn(1.0f, ox), wy0 = __fsub_rn(1.0f, oy);
+    const float ex = __fadd_rn(__fmul_rn(wy0, __fadd_rn(__fmul_rn(wx0, e00.x), __fmul_rn(ox, e10.x))),
+                               __fmul_rn(oy, __fadd_rn(__fmul_rn(wx0, e01.x), __fmul_rn(ox, e11.x))));
+    const float ey = __fadd_rn(__fmul_rn(wy0, __fadd_rn(__fmul_rn(wx0, e00.y), __fmul_rn(ox, e10.y))),
+                               __fmul_rn(oy, __fadd_rn(__fmul_rn(wx0, e01.y), __fmul_rn(ox, e11.y))));
+    ax = __fmul_rn(qm, ex);
+    ay = __fmul_rn(qm, ey);
+}
+
 // the 2D quantised deposit rule stated in slpic2d.h: the charges of the cell's nodes
 // (x, y), (x+1, y), (x, y+1), (x+1, y+1)
 __device__ __forceinline__ void quantise2d(float b, float ox, float oy, unsigned long long &q00,
@@ -289,15 +292,9 @@ __global__ void __launch_bounds__(kThreads) k_particles2d(Params2D p)
                 const float2 e00 = __ldg(p.E + k00), e10 = __ldg(p.E + k10);
                 const float2 e01 = __ldg(p.E + k00 + nx), e11 = __ldg(p.E + k10 + nx);
                 const float ox = q[k].x, oy = q[k].y;
-                const float wx0 = __fsub_rn(1.0f, ox), wy0 = __fsub_rn(1.0f, oy);
-                const float ex = __fadd_rn(
-                    __fmul_rn(wy0, __fadd_rn(__fmul_rn(wx0, e00.x), __fmul_rn(ox, e10.x))),
-                    __fmul_rn(oy, __fadd_rn(__fmul_rn(wx0, e01.x), __fmul_rn(ox, e11.x))));
-                const float ey = __fadd_rn(
-                    __fmul_rn(wy0, __fadd_rn(__fmul_rn(wx0, e00.y), __fmul_rn(ox, e10.y))),
-                    __fmul_rn(oy, __fadd_rn(__fmul_rn(wx0, e01.y), __fmul_rn(ox, e11.y))));
+                float axp, ayp;
+                accel2d(sp.qm, e00, e10, e01, e11, ox, oy, axp, ayp);
                 float vx, vy;
-                const float axp = __fmul_rn(sp.qm, ex), ayp = __fmul_rn(sp.qm, ey);
                 if (!push_v2_easy(sp.kind, q[k].z, q[k].w, z[k], axp, ayp, p.dt, sp.v0, vx, vy)) {
                     // the piece walk, here inline; counted for the diagnostics
                     namespace cg = cooperative_groups;
@@ -444,62 +441,122 @@ __device__ __forceinline__ int move2d(const Params2D &p, int cx, int cy, float o
 // particles of neighbouring cells, and each particle moves at most one cell per
 // step, so a chunk of kChunk2d consecutive slots touches a small box of the grid.
 // One CTA per chunk at a time:
-//   1. the chunk is copied into shared memory (coalesced loads), in a layout padded
-//      by one entry every 64 so that the strided reads below meet no bank conflict;
+//   1. the chunk is copied into shared memory by cp.async, 16 bytes each; a thread
+//      fills the entries that it read out for the chunk before, so no barrier lies
+//      between the two and the copies run while the window before is flushed;
 //   2. the box of its cells, relative to the cell of a live particle near its
 //      middle (x differences taken modulo nx, so a chunk that runs over the end of a
 //      row is one box), widened by the gather's node and one cell of motion;
-//   3. the window of nodes covering the box (at most kWin2d nodes) gets E copied in
-//      and its deposit cleared;
+//   3. the window of nodes covering the box (at most kWin2d nodes) gets E copied in;
 //   4. each particle is gathered, pushed, moved and deposited as k_particles2d does,
 //      from and into the window where its four nodes are inside it, else from E and
-//      into acc in global memory.  Thread (warp w, lane l) takes the chunk's
-//      particles 64 l + kPer2d w + k, so the lanes of a warp sit about a cell apart
-//      and their shared-memory atomics rarely meet on a node;
-//   5. the window's deposits go to acc (one atomic per nonzero node) and the chunk
-//      back to its slots.
+//      into acc in global memory.  Lane l of a warp takes particles of slots kSeg2d l
+//      on, so the lanes sit about a cell apart and their shared-memory atomics rarely
+//      meet on a node.  A push that needs the piece walk is left to k_hard2d: its slot
+//      goes to the step's list;
+//   5. the chunk back to its slots, the window's deposits to acc (one atomic per
+//      nonzero node) and cleared.
 // The arithmetic per particle is that of k_particles2d (the same gathered values,
 // push, move and quantised deposit), so the integer deposits and every particle are
 // the same bit for bit; only where the charge is summed first differs.
+//
+// It is bound by instruction issue (about 450 instructions a particle; its 48 bytes of HBM
+// traffic would take 475 us of the 960 at 1024^2 cells and 67 million particles), so what
+// counts is few instructions and warps that are ready to issue: seven CTAs of 128 threads
+// an SM, in different phases, rather than two of 512, which waited for each other at the
+// barriers and for their copies (issue slots used 56% -> 66% with four of 256).  Measured
+// there, with k_hard2d, a step: two CTAs of 512 threads and chunks of 2,048 1,640 us; four of
+// 256 1,440; with cp.async, the two-word window sums and the slot list 1,190; the
+// beta fixed 1,172; seven or eight of 128 and chunks of 512 1,070 (14 of 64: 1,170, the
+// windows then cost more than the waiting).  At 256^2 and 2 million 124 -> 71 us.
 // ---------------------------------------------------------------------------------
-constexpr int kT2d = 512;                        // threads per CTA
+constexpr int kT2d = 128;                        // threads per CTA
+constexpr int kTileCtas2d = 7;                   // CTAs per SM (227 KB of shared memory would hold 8)
 constexpr int kPer2d = 4;                        // particles per thread per chunk
-constexpr int kChunk2d = kT2d * kPer2d;          // 2,048 slots
-constexpr int kPad2d = kChunk2d + kChunk2d / 64; // padded shared-memory entries
-constexpr int kWin2d = 2048;                     // window nodes
+constexpr int kChunk2d = kT2d * kPer2d;          // 512 slots
+constexpr int kSeg2d = kChunk2d / 32;            // slots of a lane's segment
+constexpr int kWin2d = 768;                      // window nodes
+static_assert(kSeg2d == 16 && kChunk2d <= 1024, "vslot2d, cslot2d; the limbs' range");
 
-__device__ __forceinline__ int pad2d(int i) { return i + (i >> 6); }
+// Entries of slot j in shared memory, padded by 16 bytes a segment: a warp's 16-byte
+// reads (a segment apart) meet no bank twice; its 4-byte reads neither, as the lanes of
+// each group of eight take another of the four slots of a turn (phase 4).
+__device__ __forceinline__ int vslot2d(int j) { return j + (j >> 4); }
+__device__ __forceinline__ int cslot2d(int j) { return j + 4 * (j >> 4); }
+constexpr int kVSlots2d = kChunk2d + 32, kCSlots2d = kChunk2d + 4 * 32;
 
 size_t tile2d_smem_bytes()
 {
-    return (size_t)kPad2d * (4 + 16 + 4) + (size_t)kWin2d * (8 + 4 + 4);
+    return (size_t)kVSlots2d * 16 + (size_t)kCSlots2d * (4 + 4) + (size_t)kWin2d * (8 + 4 + 4);
 }
 
-// 64-bit integer as two 32-bit words in shared memory (value = hi 2^32 + lo, modulo
-// 2^64): the carry out of lo is detected from the old value the atomic returns
-__device__ __forceinline__ void win_add(unsigned *lo, unsigned *hi, int k, unsigned long long v)
+// The deposit rule of quantise2d in two signed words per node, value = hi 2^19 + lo: the
+// window adds them by plain 32-bit atomics, without a carry.  For 0 <= x <= 1 and
+// t = x 2^40 (exact):
+//   x 2^21 + 1.5 2^23 rounds x 2^21 to the nearest integer (the float spacing there is
+//        1), so hf, the sum less 1.5 2^23, is that integer and the sum's bits less those
+//        of 1.5 2^23 are it as an int;
+//   t - hf 2^19 is exact (|.| <= 2^18; both are multiples of the ulp of t, and at most 24
+//        bits are left), and the same addition rounds it to an integer, ties to even:
+//        rint(t), because hf 2^19 is an even integer.
+// In the differences the bits of 1.5 2^23 cancel but for node (x+1, y+1).  |lo| of a
+// deposit is at most 2^20 and a chunk adds at most 1,024 to a node: 2^30.  hi lies in
+// [-2, 2^21 + 2], so its sum lies in [-2^16, 2^32 - 2^16): win_value.
+__device__ __forceinline__ void quantise2d_limbs(float b, float ox, float oy, unsigned (&lo)[4],
+                                                 unsigned (&hi)[4])
 {
-    const unsigned vl = (unsigned)v;
-    unsigned vh = (unsigned)(v >> 32);
-    const unsigned old = atomicAdd(lo + k, vl);
-    vh += (old + vl < old) ? 1u : 0u;
-    if (vh)
-        atomicAdd(hi + k, vh);
+    const float bx = __fmul_rn(b, ox), by = __fmul_rn(b, oy), bxy = __fmul_rn(bx, oy);
+    const float x[4] = {b, bx, by, bxy};
+    unsigned l[4], h[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const float m = __fmaf_rn(x[k], 2097152.0f, 12582912.0f);
+        const float hf = __fadd_rn(m, -12582912.0f);
+        const float t = __fmul_rn(x[k], 1099511627776.0f);
+        h[k] = __float_as_uint(m);
+        l[k] = __float_as_uint(__fadd_rn(__fmaf_rn(hf, -524288.0f, t), 12582912.0f));
+    }
+    lo[0] = l[0] - l[1] - l[2] + l[3];
+    hi[0] = h[0] - h[1] - h[2] + h[3];
+    lo[1] = l[1] - l[3];
+    hi[1] = h[1] - h[3];
+    lo[2] = l[2] - l[3];
+    hi[2] = h[2] - h[3];
+    lo[3] = l[3] - 0x4B400000u;
+    hi[3] = h[3] - 0x4B400000u;
 }
 
-__global__ void __launch_bounds__(kT2d, 2) k_particles2d_tiles(Params2D p)
+// the value of a node's summed words
+__device__ __forceinline__ unsigned long long win_value(unsigned lo, unsigned hi)
+{
+    const long long h = (long long)(hi + 65536u) - 65536;
+    return (unsigned long long)(h * 524288 + (long long)(int)lo);
+}
+
+__device__ __forceinline__ void cp_async16(void *dst, const void *src, int bytes)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(dst)),
+                 "l"(src), "r"(bytes)
+                 : "memory");
+}
+
+template <int kKind>
+__global__ void __launch_bounds__(kT2d, kTileCtas2d) k_particles2d_tiles(const __grid_constant__ Params2D p)
 {
     extern __shared__ __align__(16) unsigned char smem2d[];
-    float4 *s_v = reinterpret_cast<float4 *>(smem2d);                  // [kPad2d]
-    float2 *s_E = reinterpret_cast<float2 *>(s_v + kPad2d);            // [kWin2d]
-    int32_t *s_c = reinterpret_cast<int32_t *>(s_E + kWin2d);          // [kPad2d]
-    float *s_z = reinterpret_cast<float *>(s_c + kPad2d);              // [kPad2d]
-    unsigned *s_lo = reinterpret_cast<unsigned *>(s_z + kPad2d);       // [kWin2d]
+    float4 *s_v = reinterpret_cast<float4 *>(smem2d);                  // [kVSlots2d]
+    float2 *s_E = reinterpret_cast<float2 *>(s_v + kVSlots2d);         // [kWin2d]
+    int32_t *s_c = reinterpret_cast<int32_t *>(s_E + kWin2d);          // [kCSlots2d]
+    float *s_z = reinterpret_cast<float *>(s_c + kCSlots2d);           // [kCSlots2d]
+    unsigned *s_lo = reinterpret_cast<unsigned *>(s_z + kCSlots2d);    // [kWin2d]
     unsigned *s_hi = s_lo + kWin2d;                                    // [kWin2d]
-    __shared__ int s_ref, s_box[4];  // reference cell; min dx, -max dx, min dy, -max dy
+    __shared__ int s_ref, s_box[2][4];  // reference cell; min dx, -max dx, min dy, -max dy
     __shared__ unsigned s_abs[2];
+    __shared__ int s_nh;                         // the chunk's walked pushes: their number
+    __shared__ unsigned short s_list[kChunk2d];  // and places
 
-    const int s = blockIdx.y;
+    const int s = blockIdx.y, tid = threadIdx.x;
     const Species2D &sp = p.sp[s];
     const long long step = *(volatile long long *)&p.st->step;
     const int P = (int)(step & 1);
@@ -512,54 +569,74 @@ __global__ void __launch_bounds__(kT2d, 2) k_particles2d_tiles(Params2D p)
     float *__restrict__ zout = sp.vz[P ^ 1];
     unsigned long long *acc = p.acc + (size_t)s * p.nn;
     const int nx = p.nx, ny = p.ny;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    if (threadIdx.x < 2)
-        s_abs[threadIdx.x] = 0u;
+    const int lane = tid & 31, warp = tid >> 5;
+    const float qm = sp.qm, v0 = sp.v0, dt = p.dt;
+    const int kind = kKind < 0 ? sp.kind : kKind;
+    for (int k = tid; k < kWin2d; k += kT2d) {
+        s_lo[k] = 0u;
+        s_hi[k] = 0u;
+    }
+    if (tid < 8)
+        s_box[tid >> 2][tid & 3] = INT_MAX;
+    if (tid < 2)
+        s_abs[tid] = 0u;
+    if (tid == 0)
+        s_nh = 0;
+    __syncthreads();
     unsigned na0 = 0, na1 = 0;
 
+    // ---- 1. a chunk into shared memory: this thread's four cells and vz (slots 4 tid on)
+    // and its four of every kT2d (ox, oy, vx, vy); returns the cell of the middle slot
+    auto load = [&](long long base, int cnt) -> int {
+        const int left = cnt - 4 * tid;
+        if (left > 0) {
+            const int bytes = 4 * min(left, 4);
+            cp_async16(s_c + cslot2d(4 * tid), cin + base + 4 * tid, bytes);
+            cp_async16(s_z + cslot2d(4 * tid), zin + base + 4 * tid, bytes);
+        }
+#pragma unroll
+        for (int i = 0; i < kPer2d; ++i) {
+            const int j = tid + i * kT2d;
+            if (j < cnt)
+                cp_async16(s_v + vslot2d(j), vin + base + j, 16);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+        return __ldcs(cin + base + cnt / 2);
+    };
+
     const long long nchunks = (n + kChunk2d - 1) / kChunk2d;
-    for (long long ch = blockIdx.x; ch < nchunks; ch += gridDim.x) {
+    int ref_next = -1, turn = 0;
+    if (blockIdx.x < nchunks)
+        ref_next = load((long long)blockIdx.x * kChunk2d,
+                        (int)min((long long)kChunk2d, n - (long long)blockIdx.x * kChunk2d));
+    for (long long ch = blockIdx.x; ch < nchunks; ch += gridDim.x, turn ^= 1) {
         const long long base = ch * kChunk2d;
         const int cnt = (int)min((long long)kChunk2d, n - base);
-        // ---- 1. the chunk into shared memory
-        for (int j = threadIdx.x; j < kChunk2d; j += kT2d) {
-            const int q = pad2d(j);
-            if (j < cnt) {
-                s_c[q] = __ldcs(cin + base + j);
-                s_v[q] = __ldcs(vin + base + j);
-                s_z[q] = __ldcs(zin + base + j);
-            } else {
-                s_c[q] = -1;
-            }
-        }
-        if (threadIdx.x == 0) {
-            s_box[0] = s_box[1] = s_box[2] = s_box[3] = INT_MAX;
-            s_ref = -1;
-        }
-        __syncthreads();
-        // ---- 2. the reference cell (a live particle at or after the middle, else
-        // before it) and the box of the chunk's cells relative to it
-        if (threadIdx.x == 0) {
-            int r = -1;
-            for (int j = cnt / 2; j < cnt && r < 0; ++j)
-                r = s_c[pad2d(j)];
-            for (int j = cnt / 2 - 1; j >= 0 && r < 0; --j)
-                r = s_c[pad2d(j)];
-            s_ref = r;
-        }
-        __syncthreads();
-        const int ref = s_ref;
-        if (ref < 0) {  // nothing live: the holes stay holes
-            for (int j = threadIdx.x; j < cnt; j += kT2d)
-                __stcs(cout + base + j, -1);
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        // ---- 2. the reference cell (the middle slot's; if that is a hole, a live particle
+        // after it, else before it) and the box of the chunk's cells relative to it
+        int ref = ref_next;
+        if (ref < 0) {
             __syncthreads();
-            continue;
+            if (tid == 0) {
+                int r = -1;
+                for (int j = cnt / 2; j < cnt && r < 0; ++j)
+                    r = s_c[cslot2d(j)];
+                for (int j = cnt / 2 - 1; j >= 0 && r < 0; --j)
+                    r = s_c[cslot2d(j)];
+                s_ref = r;
+            }
+            __syncthreads();
+            ref = s_ref;  // < 0: nothing live; the box is empty and phase 4 finds no particle
         }
-        const int ry = div_nx(p, ref), rx = ref - ry * nx;
+        const int ry = ref < 0 ? 0 : div_nx(p, ref), rx = ref < 0 ? 0 : ref - ry * nx;
         {
             int mnx = INT_MAX, mxx = INT_MAX, mny = INT_MAX, mxy = INT_MAX;  // max as -min
-            for (int k = 0; k < kPer2d; ++k) {
-                const int c = s_c[pad2d(k * kT2d + threadIdx.x)];
+            const int4 c4 = *reinterpret_cast<const int4 *>(s_c + cslot2d(4 * tid));
+            const int cc[4] = {c4.x, c4.y, c4.z, c4.w};
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+                const int c = 4 * tid + k < cnt ? cc[k] : -1;
                 if (c >= 0) {
                     const int cy = div_nx(p, c);
                     int dx = c - cy * nx - rx;  // to [-nx/2, nx/2)
@@ -579,53 +656,54 @@ __global__ void __launch_bounds__(kT2d, 2) k_particles2d_tiles(Params2D p)
             mny = __reduce_min_sync(0xffffffffu, mny);
             mxy = __reduce_min_sync(0xffffffffu, mxy);
             if (lane == 0) {
-                atomicMin(&s_box[0], mnx);
-                atomicMin(&s_box[1], mxx);
-                atomicMin(&s_box[2], mny);
-                atomicMin(&s_box[3], mxy);
+                atomicMin(&s_box[turn][0], mnx);
+                atomicMin(&s_box[turn][1], mxx);
+                atomicMin(&s_box[turn][2], mny);
+                atomicMin(&s_box[turn][3], mxy);
             }
         }
-        __syncthreads();
+        __syncthreads();  // the box, and the whole chunk in place
         // ---- 3. the window: node columns wx0 .. wx0+ww-1 (modulo nx), rows wy0 ..
         // wy0+wh-1, covering the box widened by the gather's node and one cell of
         // motion each way (cut to kWin2d nodes; particles outside it go to global memory)
-        int ww = (-s_box[1]) - s_box[0] + 4;
-        int wx0 = rx + s_box[0] - 1;
-        const int wy0 = max(0, ry + s_box[2] - 1);
-        int wh = min(ny, ry - s_box[3] + 2) - wy0 + 1;
-        if (ww >= nx) {
-            ww = nx;
-            wx0 = 0;
+        int ww = 0, wx0 = 0, wy0 = 0, wh = 0;
+        if (ref >= 0) {
+            const int *box = s_box[turn];
+            ww = (-box[1]) - box[0] + 4;
+            wx0 = rx + box[0] - 1;
+            wy0 = max(0, ry + box[2] - 1);
+            wh = min(ny, ry - box[3] + 2) - wy0 + 1;
+            if (ww >= nx) {
+                ww = nx;
+                wx0 = 0;
+            }
+            wx0 %= nx;
+            if (wx0 < 0)
+                wx0 += nx;
+            if (ww > kWin2d / 2)
+                ww = kWin2d / 2;
+            if (ww * wh > kWin2d)
+                wh = kWin2d / ww;
         }
-        wx0 %= nx;
-        if (wx0 < 0)
-            wx0 += nx;
-        if (ww > kWin2d / 2)
-            ww = kWin2d / 2;
-        if (ww * wh > kWin2d)
-            wh = kWin2d / ww;
+        if (tid < 4)
+            s_box[turn ^ 1][tid] = INT_MAX;
         // a warp per window row, a lane per column
         for (int iy = warp; iy < wh; iy += kT2d / 32) {
             const float2 *Er = p.E + (size_t)(wy0 + iy) * nx;
-            for (int ix = lane; ix < ww; ix += 32) {
-                const int gx = wx0 + ix < nx ? wx0 + ix : wx0 + ix - nx;
-                const int k = iy * ww + ix;
-                s_E[k] = __ldg(Er + gx);
-                s_lo[k] = 0u;
-                s_hi[k] = 0u;
-            }
+            for (int ix = lane; ix < ww; ix += 32)
+                s_E[iy * ww + ix] = __ldg(Er + (wx0 + ix < nx ? wx0 + ix : wx0 + ix - nx));
         }
         __syncthreads();
-        // ---- 4. the particles, lanes of a warp 64 slots apart
+        // ---- 4. the particles, lanes of a warp a segment apart
 #pragma unroll 1
         for (int k = 0; k < kPer2d; ++k) {
-            const int j = lane * 64 + warp * kPer2d + k;
-            const int q = pad2d(j);
-            const int c = j < cnt ? s_c[q] : -1;
+            const int j = lane * kSeg2d + warp * kPer2d + ((k + (lane >> 3)) & 3);
+            const int qc = cslot2d(j), qv = vslot2d(j);
+            const int c = j < cnt ? s_c[qc] : -1;
             if (c < 0)
                 continue;
-            const float4 pv = s_v[q];
-            const float z = s_z[q];
+            const float4 pv = s_v[qv];
+            const float z = s_z[qc];
             const int cy = div_nx(p, c), cx = c - cy * nx;
             int ix = cx - wx0;
             if (ix < 0)
@@ -639,102 +717,114 @@ __global__ void __launch_bounds__(kT2d, 2) k_particles2d_tiles(Params2D p)
                 e01 = s_E[k00 + ww];
                 e11 = s_E[k00 + ww + 1];
             } else {
-                const int cx1 = (cx + 1 == nx) ? 0 : cx + 1;
-                const int k00 = cy * nx + cx, k10 = cy * nx + cx1;
-                e00 = __ldg(p.E + k00);
+                const int k10 = (cx + 1 == nx) ? c + 1 - nx : c + 1;
+                e00 = __ldg(p.E + c);
                 e10 = __ldg(p.E + k10);
-                e01 = __ldg(p.E + k00 + nx);
+                e01 = __ldg(p.E + c + nx);
                 e11 = __ldg(p.E + k10 + nx);
             }
-            const float ox = pv.x, oy = pv.y;
-            const float wx0f = __fsub_rn(1.0f, ox), wy0f = __fsub_rn(1.0f, oy);
-            const float ex = __fadd_rn(
-                __fmul_rn(wy0f, __fadd_rn(__fmul_rn(wx0f, e00.x), __fmul_rn(ox, e10.x))),
-                __fmul_rn(oy, __fadd_rn(__fmul_rn(wx0f, e01.x), __fmul_rn(ox, e11.x))));
-            const float ey = __fadd_rn(
-                __fmul_rn(wy0f, __fadd_rn(__fmul_rn(wx0f, e00.y), __fmul_rn(ox, e10.y))),
-                __fmul_rn(oy, __fadd_rn(__fmul_rn(wx0f, e01.y), __fmul_rn(ox, e11.y))));
-            const float axp = __fmul_rn(sp.qm, ex), ayp = __fmul_rn(sp.qm, ey);
+            float axp, ayp;
+            accel2d(qm, e00, e10, e01, e11, pv.x, pv.y, axp, ayp);
             float vx, vy;
-            if (!push_v2_easy(sp.kind, pv.z, pv.w, z, axp, ayp, p.dt, sp.v0, vx, vy)) {
-                // the piece walk: listed for k_hard2d, which pushes it and writes its
-                // slot (pushed here once the list is full)
-                namespace cg = cooperative_groups;
-                cg::coalesced_group g = cg::coalesced_threads();
-                unsigned long long hb = 0;
-                if (g.thread_rank() == 0)
-                    hb = atomicAdd(&p.st->hard_n[s], (unsigned long long)g.size());
-                hb = g.shfl(hb, 0) + g.thread_rank();
-                if ((long long)hb < sp.hard_cap) {
-                    int4 *r = reinterpret_cast<int4 *>(sp.hard + hb);
-                    r[0] = make_int4((int)(base + j), c, __float_as_int(axp), __float_as_int(ayp));
-                    r[1] = make_int4(__float_as_int(pv.x), __float_as_int(pv.y),
-                                     __float_as_int(pv.z), __float_as_int(pv.w));
-                    r[2] = make_int4(__float_as_int(z), 0, 0, 0);
-                    s_c[q] = -2;  // its slot is k_hard2d's
-                    continue;
-                }
-                push_v2(sp.kind, pv.z, pv.w, z, axp, ayp, p.dt, sp.v0, vx, vy);
+            if (!push_v2_easy(kind, pv.z, pv.w, z, axp, ayp, dt, v0, vx, vy)) {
+                // the piece walk: k_hard2d pushes it and writes its slot
+                s_list[atomicAdd(&s_nh, 1)] = (unsigned short)j;
+                continue;
             }
             // x^{n+1} = x^n + beta(|v^{n+1/2}|) v^{n+1/2} dt, in cell units
-            const float b = beta_q(sp.kind, vx, vy, z, sp.v0);
+            const float b = beta_q(kind, vx, vy, z, v0);
             int ncx, ncy;
             float dxn, dyn;
-            const int wall = move2d(p, cx, cy, ox, oy, vx, vy, b, ncx, ncy, dxn, dyn);
-            if (wall == 0) {
-                ++na0;
-                s_c[q] = -1;
-            } else if (wall == 1) {
-                ++na1;
-                s_c[q] = -1;
+            const int wall = move2d(p, cx, cy, pv.x, pv.y, vx, vy, b, ncx, ncy, dxn, dyn);
+            if (wall >= 0) {
+                if (wall == 0)
+                    ++na0;
+                else
+                    ++na1;
+                s_c[qc] = -1;
+                continue;
+            }
+            s_c[qc] = ncy * nx + ncx;
+            s_v[qv] = make_float4(dxn, dyn, vx, vy);
+            int nix = ncx - wx0;
+            if (nix < 0)
+                nix += nx;
+            const int niy = ncy - wy0;
+            if (nix <= ww - 2 && niy >= 0 && niy <= wh - 2) {
+                unsigned lo[4], hi[4];
+                quantise2d_limbs(b, dxn, dyn, lo, hi);
+                unsigned *w0 = s_lo + niy * ww + nix, *w1 = w0 + ww;
+                atomicAdd(w0, lo[0]);
+                atomicAdd(w0 + kWin2d, hi[0]);
+                atomicAdd(w0 + 1, lo[1]);
+                atomicAdd(w0 + kWin2d + 1, hi[1]);
+                atomicAdd(w1, lo[2]);
+                atomicAdd(w1 + kWin2d, hi[2]);
+                atomicAdd(w1 + 1, lo[3]);
+                atomicAdd(w1 + kWin2d + 1, hi[3]);
             } else {
-                unsigned long long q00, q10, q01, q11;
-                quantise2d(b, dxn, dyn, q00, q10, q01, q11);
-                int nix = ncx - wx0;
-                if (nix < 0)
-                    nix += nx;
-                const int niy = ncy - wy0;
-                if (nix <= ww - 2 && niy >= 0 && niy <= wh - 2) {
-                    const int k00 = niy * ww + nix;
-                    win_add(s_lo, s_hi, k00, q00);
-                    win_add(s_lo, s_hi, k00 + 1, q10);
-                    win_add(s_lo, s_hi, k00 + ww, q01);
-                    win_add(s_lo, s_hi, k00 + ww + 1, q11);
-                } else {
-                    const int ncx1 = (ncx + 1 == nx) ? 0 : ncx + 1;
-                    const int m00 = ncy * nx + ncx, m10 = ncy * nx + ncx1;
-                    atomicAdd(acc + m00, q00);
-                    atomicAdd(acc + m10, q10);
-                    atomicAdd(acc + m00 + nx, q01);
-                    atomicAdd(acc + m10 + nx, q11);
-                }
-                s_c[q] = ncy * nx + ncx;
-                s_v[q] = make_float4(dxn, dyn, vx, vy);
+                const int m00 = ncy * nx + ncx, m10 = (ncx + 1 == nx) ? m00 + 1 - nx : m00 + 1;
+                deposit2d(acc, m00, m10, m00 + nx, m10 + nx, b, dxn, dyn);
             }
         }
         __syncthreads();
-        // ---- 5. the window's deposits to acc, the chunk to its slots
+        // ---- 5. the walked pushes to the list (their slots' contents here are overwritten
+        // by k_hard2d), the chunk to its slots, the next chunk's copies, the window
+        if (warp == 0) {
+            const int nh = s_nh;
+            if (nh) {
+                unsigned long long hb = 0;
+                if (lane == 0)
+                    hb = atomicAdd(&p.st->hard_n[s], (unsigned long long)nh);
+                hb = __shfl_sync(0xffffffffu, hb, 0);
+                for (int i = lane; i < nh; i += 32)
+                    sp.hard[hb + i] = (int32_t)(base + s_list[i]);
+                if (lane == 0)
+                    s_nh = 0;
+            }
+        }
+        {
+            const int4 c4 = *reinterpret_cast<const int4 *>(s_c + cslot2d(4 * tid));
+            const float4 z4 = *reinterpret_cast<const float4 *>(s_z + cslot2d(4 * tid));
+            const long long o = base + 4 * tid;
+            const int left = cnt - 4 * tid;
+            if (left >= 4) {
+                __stcs(reinterpret_cast<int4 *>(cout + o), c4);
+                __stcs(reinterpret_cast<float4 *>(zout + o), z4);
+            } else if (left > 0) {
+                __stcs(cout + o, c4.x);
+                __stcs(zout + o, z4.x);
+                if (left > 1) {
+                    __stcs(cout + o + 1, c4.y);
+                    __stcs(zout + o + 1, z4.y);
+                }
+                if (left > 2) {
+                    __stcs(cout + o + 2, c4.z);
+                    __stcs(zout + o + 2, z4.z);
+                }
+            }
+#pragma unroll
+            for (int i = 0; i < kPer2d; ++i) {
+                const int j = tid + i * kT2d;
+                if (j < cnt)
+                    __stcs(vout + base + j, s_v[vslot2d(j)]);
+            }
+        }
+        if (ch + gridDim.x < nchunks) {
+            const long long nb = (ch + gridDim.x) * kChunk2d;
+            ref_next = load(nb, (int)min((long long)kChunk2d, n - nb));
+        }
         for (int iy = warp; iy < wh; iy += kT2d / 32) {
             unsigned long long *ar = acc + (size_t)(wy0 + iy) * nx;
             for (int ix = lane; ix < ww; ix += 32) {
                 const int k = iy * ww + ix;
-                const unsigned long long v = ((unsigned long long)s_hi[k] << 32) + s_lo[k];
+                const unsigned long long v = win_value(s_lo[k], s_hi[k]);
+                s_lo[k] = 0u;
+                s_hi[k] = 0u;
                 if (v)
                     atomicAdd(ar + (wx0 + ix < nx ? wx0 + ix : wx0 + ix - nx), v);
             }
         }
-        for (int j = threadIdx.x; j < cnt; j += kT2d) {
-            const int q = pad2d(j);
-            const int c = s_c[q];
-            if (c == -2)
-                continue;  // listed for k_hard2d
-            __stcs(cout + base + j, c);
-            if (c >= 0) {
-                __stcs(vout + base + j, s_v[q]);
-                __stcs(zout + base + j, s_z[q]);
-            }
-        }
-        __syncthreads();
     }
     na0 = __reduce_add_sync(0xffffffffu, na0);
     na1 = __reduce_add_sync(0xffffffffu, na1);
@@ -745,11 +835,23 @@ __global__ void __launch_bounds__(kT2d, 2) k_particles2d_tiles(Params2D p)
             atomicAdd(&s_abs[1], na1);
     }
     __syncthreads();
-    if (threadIdx.x < 2 && s_abs[threadIdx.x])
-        atomicAdd(&p.st->absorbed_step[s][threadIdx.x], (unsigned long long)s_abs[threadIdx.x]);
+    if (tid < 2 && s_abs[tid])
+        atomicAdd(&p.st->absorbed_step[s][tid], (unsigned long long)s_abs[tid]);
 }
 
-// The particles the tile kernel listed: the full push (series or piece walk, the
+// The instantiation for a simulation's species: the Heaviside beta fixed at compile time
+// where all have it, else read per species (the same arithmetic).
+typedef void (*TileKernel)(Params2D);
+
+TileKernel tile_kernel(const Params2D &p)
+{
+    for (int s = 0; s < p.ns; ++s)
+        if (p.sp[s].kind != SLPIC_BETA_HEAVISIDE)
+            return k_particles2d_tiles<-1>;
+    return k_particles2d_tiles<SLPIC_BETA_HEAVISIDE>;
+}
+
+// The particles the tile kernel listed: gathered again, the full push (series or piece walk, the
 // arithmetic of the inline push), the move, the plates and the deposit by global
 // atomics; each writes its own slot.  The species' lists are one index space.
 __global__ void __launch_bounds__(256) k_hard2d(Params2D p)
@@ -765,7 +867,7 @@ __global__ void __launch_bounds__(256) k_hard2d(Params2D p)
 #pragma unroll
     for (int s = 0; s < kMaxS; ++s) {
         const long long n = s < p.ns ? (long long)*(volatile unsigned long long *)&p.st->hard_n[s] : 0;
-        pre[s + 1] = pre[s] + (s < p.ns ? min(n, p.sp[s].hard_cap) : 0);
+        pre[s + 1] = pre[s] + n;
     }
     const long long total = pre[kMaxS];
     for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -779,19 +881,21 @@ __global__ void __launch_bounds__(256) k_hard2d(Params2D p)
                 i0 = pre[r];
             }
         const Species2D &sp = p.sp[s];
-        const int4 *rec = reinterpret_cast<const int4 *>(sp.hard + (t - i0));
-        const int4 r0 = __ldcs(rec), r1 = __ldcs(rec + 1), r2 = __ldcs(rec + 2);
-        const int slot = r0.x, c = r0.y;
-        const float ax = __int_as_float(r0.z), ay = __int_as_float(r0.w);
-        const float ox = __int_as_float(r1.x), oy = __int_as_float(r1.y);
-        const float ux = __int_as_float(r1.z), uy = __int_as_float(r1.w), z = __int_as_float(r2.x);
-        float vx, vy;
-        push_v2(sp.kind, ux, uy, z, ax, ay, p.dt, sp.v0, vx, vy);
-        const float b = beta_q(sp.kind, vx, vy, z, sp.v0);
+        const int slot = __ldcs(sp.hard + (t - i0));
+        const int c = sp.cell[P][slot];
+        const float4 q = sp.pv[P][slot];
+        const float z = sp.vz[P][slot];
         const int cy = div_nx(p, c), cx = c - cy * p.nx;
+        const int k10 = (cx + 1 == p.nx) ? c + 1 - p.nx : c + 1;
+        float ax, ay;
+        accel2d(sp.qm, __ldg(p.E + c), __ldg(p.E + k10), __ldg(p.E + c + p.nx),
+                __ldg(p.E + k10 + p.nx), q.x, q.y, ax, ay);
+        float vx, vy;
+        push_v2(sp.kind, q.z, q.w, z, ax, ay, p.dt, sp.v0, vx, vy);
+        const float b = beta_q(sp.kind, vx, vy, z, sp.v0);
         int ncx, ncy;
         float dxn, dyn;
-        const int wall = move2d(p, cx, cy, ox, oy, vx, vy, b, ncx, ncy, dxn, dyn);
+        const int wall = move2d(p, cx, cy, q.x, q.y, vx, vy, b, ncx, ncy, dxn, dyn);
         if (wall >= 0) {
             atomicAdd(&s_abs[s][wall], 1u);
             sp.cell[P ^ 1][slot] = -1;
@@ -1971,7 +2075,8 @@ struct slpic2d_sim {
     Params2D p{};
     int ctas = 1;     // particle-kernel CTAs per species
     int tile_ctas = 0;  // k_particles2d_tiles CTAs per species (0: not resident)
-    int small_ctas = 1; // k_hard2d and k_inject2d: 2 CTAs of 256 threads per SM
+    int hard_ctas = 1;  // k_hard2d: all resident
+    int small_ctas = 1; // k_inject2d: 2 CTAs of 256 threads per SM
     bool prepared = false;
     bool timing = false;               // record events around the kernels of each step
     std::vector<cudaEvent_t> events;   // 4 per recorded step
@@ -2241,13 +2346,9 @@ extern "C" int slpic2d_create(const slpic2d_config *c, slpic2d_t **out)
             ok = alloc((void **)&d.cell[b], sizeof(int32_t) * sp.capacity) &&
                  alloc((void **)&d.pv[b], sizeof(float4) * sp.capacity) &&
                  alloc((void **)&d.vz[b], sizeof(float) * sp.capacity);
-        // the step's list of walked pushes: an eighth of the capacity, at least 64k
-        // (slot indices are int32; beyond the list the tile kernel pushes inline)
-        d.hard_cap = sp.capacity <= INT_MAX
-                         ? std::min<long long>(sp.capacity, std::max<long long>(sp.capacity / 8, 65536))
-                         : 0;
-        if (ok && d.hard_cap)
-            ok = alloc((void **)&d.hard, sizeof(HardRec2D) * d.hard_cap);
+        // the slots of a step's walked pushes (all of them, at most)
+        if (ok)
+            ok = alloc((void **)&d.hard, sizeof(int32_t) * sp.capacity);
         d.capacity = sp.capacity;
         d.qm = (float)(sp.q / sp.m);
         d.v0 = (float)sp.v0;
@@ -2269,15 +2370,18 @@ extern "C" int slpic2d_create(const slpic2d_config *c, slpic2d_t **out)
         return bail(SLPIC_ERR_CUDA, "CG kernel occupancy query failed");
     h->ctas = sms * 4;
     h->small_ctas = sms * 2;
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_hard2d, 256, 0) != cudaSuccess || occ < 1)
+        return bail(SLPIC_ERR_CUDA, "kernel occupancy query failed");
+    h->hard_ctas = sms * occ;
     {
         // the tile kernel: every CTA of both species resident at once
         int occ_t = 0;
-        if (cudaFuncSetAttribute(k_particles2d_tiles, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        if (cudaFuncSetAttribute(tile_kernel(p), cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)tile2d_smem_bytes()) == cudaSuccess &&
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_t, k_particles2d_tiles, kT2d,
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ_t, tile_kernel(p), kT2d,
                                                           tile2d_smem_bytes()) == cudaSuccess &&
             occ_t > 0)
-            h->tile_ctas = std::max(1, sms * occ_t / p.ns);
+            h->tile_ctas = std::max(1, sms * std::min(occ_t, kTileCtas2d) / p.ns);
         cudaGetLastError();
     }
     if (!alloc((void **)&p.part, sizeof(double) * 3 * p.cg_v))
@@ -2494,8 +2598,8 @@ extern "C" int slpic2d_step(slpic2d_t *h, int64_t nsteps)
         if (compact)
             k_particles2d<true><<<dim3(h->ctas, p.ns), kThreads, 0, h->stream>>>(p);
         else if (h->tile_ctas) {
-            k_particles2d_tiles<<<dim3(h->tile_ctas, p.ns), kT2d, tile2d_smem_bytes(), h->stream>>>(p);
-            k_hard2d<<<h->small_ctas, 256, 0, h->stream>>>(p);
+            tile_kernel(p)<<<dim3(h->tile_ctas, p.ns), kT2d, tile2d_smem_bytes(), h->stream>>>(p);
+            k_hard2d<<<h->hard_ctas, 256, 0, h->stream>>>(p);
         } else {
             k_particles2d<false><<<dim3(h->ctas, p.ns), kThreads, 0, h->stream>>>(p);
         }
