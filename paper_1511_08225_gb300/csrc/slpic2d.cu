@@ -88,6 +88,7 @@ struct Params2D {
     int nx_s;
     float dt, dt_dx;
     double dx, dt64, k2;          // k2 = dx^2 / eps0
+    double half_dx;               // 0.5 / dx
     double phi_lo, phi_hi, rtol2;  // rtol^2
     int cg_maxit;
     int src_mode, src_ref;
@@ -109,6 +110,7 @@ struct Params2D {
     double *inv_m;            // [nn] Thomas multipliers 1/m_j per (row j, mode k)
     double *seg_f, *seg_b;    // [nn] their products within a segment, up to / from row j
     double *rpart;            // [2 (ny+1)] per-row sums of r^2 and b^2
+    unsigned *finished;       // CTAs of k_fft_finish that have written theirs
     int *hist, *cursor, *bsum;  // cell sort: counts per cell, then slots; block sums
 };
 
@@ -1287,14 +1289,14 @@ __device__ __forceinline__ void store_E(const Params2D &p, int idx)
     const int ip = (i + 1 == nx) ? idx + 1 - nx : idx + 1;
     const int im = (i == 0) ? idx - 1 + nx : idx - 1;
     const double *f = p.phi;
-    const double ex = -(__ldcg(f + ip) - __ldcg(f + im)) * (0.5 / p.dx);
+    const double ex = -(__ldcg(f + ip) - __ldcg(f + im)) * p.half_dx;
     double ey;
     if (j == 0)
         ey = -(__ldcg(f + idx + nx) - __ldcg(f + idx)) / p.dx;
     else if (j == ny)
         ey = -(__ldcg(f + idx) - __ldcg(f + idx - nx)) / p.dx;
     else
-        ey = -(__ldcg(f + idx + nx) - __ldcg(f + idx - nx)) * (0.5 / p.dx);
+        ey = -(__ldcg(f + idx + nx) - __ldcg(f + idx - nx)) * p.half_dx;
     p.E[idx] = make_float2((float)ex, (float)ey);
 }
 
@@ -1582,32 +1584,168 @@ int cg_grid(const Params2D &p)
 // The 5-point system A phi = b on the interior rows j = 1..ny-1 is periodic in x,
 // so the discrete Fourier transform along x diagonalises its x part: mode k of row
 // j obeys (4 - 2 cos(2 pi k/nx)) u_j - u_{j-1} - u_{j+1} = b^_j with u_0 = u_ny = 0
-// (the plate potentials are in b).  Three passes: a forward radix-2 FFT per row
-// (one CTA per row, the row in shared memory, FP64), the Thomas algorithm per mode
-// (one thread per k, the multipliers tabulated at creation), the inverse FFT per
+// (the plate potentials are in b).  Three passes, in FP64: a forward FFT per row, the
+// Thomas algorithm per mode (the multipliers tabulated at creation), the inverse FFT per
 // row.  Then E and the true residual as for the CG.
-constexpr int kFftThreads = 256;
+//
+// The arithmetic is that of a complex radix-2 transform (decimation in time) with unfused
+// butterflies, of Thomas in 32 segments, to the last bit: what a wall absorbs turns on E's
+// last bits, so a transform that rounds otherwise (of half the length, with fused
+// multiply-adds: 166 us at 1,024^2) would change every run.  The FP64 pipe (2 lanes an SM)
+// bounds the large grids: some 40 thousand instructions a row of 1,024 each way.  Small
+// grids are bound by latency, so a thread keeps its points in registers over several levels
+// of butterflies and the row's threads meet in shared memory only between those, twiddles and
+// coefficients straight from L2 to registers.  The solve of a step (with the residual's report, a
+// launch of its own before): 1,024^2 445 -> 299 us (the rows 117 us, 77% of the FP64 pipe),
+// 256^2 73 -> 52.
+constexpr int kFftMaxThreads = 512;
+constexpr int kFinishThreads = 128;
 
-// in-place radix-2 FFT of x[0..n) held in bit-reversed order; sign -1 forward,
-// +1 inverse (unnormalised)
-__device__ void fft_smem(double2 *x, const double2 *__restrict__ tw, int n, double sign)
+// Levels of butterflies that a thread does between two meetings, on 2^levels points: 3, or
+// 1 where that leaves fewer than 512 warps (3 an SM), too few to hide the FP64 latency.  The
+// solve of a step with 1 and with 3: 64 x 64 37.2 and 45.4 us, 64 x 1,000 (250 warps with 3)
+// 59.6 and 65.3, 256^2 52.4 and 57.8, 512^2 (1,022) 104.5 and 93.9, 1,024^2 316 and 299.
+int fft_levels(int nx, int ny)
 {
-    for (int len = 2; len <= n; len <<= 1) {
-        const int half = len >> 1, step = n / len;
-        __syncthreads();
-        for (int b = threadIdx.x; b < n / 2; b += blockDim.x) {
-            const int g = b / half, pos = b - g * half;
-            const int i0 = g * len + pos, i1 = i0 + half;
-            const double2 w = tw[pos * step];
-            const double wr = w.x, wi = sign * w.y;
-            const double2 v = x[i1];
-            const double tr = wr * v.x - wi * v.y, ti = wr * v.y + wi * v.x;
-            const double2 u = x[i0];
-            x[i0] = make_double2(u.x + tr, u.y + ti);
-            x[i1] = make_double2(u.x - tr, u.y - ti);
+    return ((long long)(ny - 1) * nx >> 8) < 512 ? 1 : 3;
+}
+// threads of a row's transform, and rows of a CTA (a warp at least)
+__host__ __device__ __forceinline__ int fft_row_threads(int nx, int levels)
+{
+    const int T = nx >> levels ? nx >> levels : 1;
+    return T < kFftMaxThreads ? T : kFftMaxThreads;
+}
+__host__ __device__ __forceinline__ int fft_cta_rows(int nx, int levels)
+{
+    const int T = fft_row_threads(nx, levels);
+    return T < 32 ? 32 / T : 1;
+}
+
+// Place of point i of a row in shared memory: the low three bits of the place are mixed
+// with the bits above, so that eight threads meet eight different 16-byte banks whichever
+// three bits of i tell them apart.  Linear: the place of a sum of numbers without a bit in
+// common is the exclusive or of theirs.
+__device__ __forceinline__ int fft_place(int i) { return i ^ (((i >> 3) ^ (i >> 6) ^ (i >> 9)) & 7); }
+
+// (u, v) -> (u + w v, u - w v), w = (wr, wi)
+__device__ __forceinline__ void butterfly(double2 &u, double2 &v, double wr, double wi)
+{
+    const double tr = wr * v.x - wi * v.y, ti = wr * v.y + wi * v.x;
+    const double2 a = u;
+    u = make_double2(a.x + tr, a.y + ti);
+    v = make_double2(a.x - tr, a.y - ti);
+}
+// w = 1
+__device__ __forceinline__ void butterfly1(double2 &u, double2 &v)
+{
+    const double2 a = u, b = v;
+    u = make_double2(a.x + b.x, a.y + b.y);
+    v = make_double2(a.x - b.x, a.y - b.y);
+}
+
+// R levels from the first (points a unit apart; w: the tabulated eighths of a turn)
+template <int R, bool INV>
+__device__ __forceinline__ void first_levels(double2 *z, const double2 (&w)[4])
+{
+#pragma unroll
+    for (int d = 0; d < R; ++d)
+#pragma unroll
+        for (int r = 0; r < (1 << R); ++r)
+            if (!(r >> d & 1)) {
+                const int e = (r & ((1 << d) - 1)) << (2 - d);
+                if (e == 0)
+                    butterfly1(z[r], z[r + (1 << d)]);
+                else if (INV || d == 2)
+                    butterfly(z[r], z[r + (1 << d)], w[e].x, INV ? w[e].y : -w[e].y);
+                else {  // forward, the second level: both points are real
+                    const double u = z[r].x, v = z[r + 2].x, tr = w[e].x * v, ti = -w[e].y * v;
+                    z[r] = make_double2(u + tr, ti);
+                    z[r + 2] = make_double2(u - tr, -ti);
+                }
+            }
+}
+
+// LV levels from points h apart; lo the first point's place among the h
+template <int LV, bool INV>
+__device__ __forceinline__ void more_levels(double2 *z, const double2 *__restrict__ tw, int nx, int lo,
+                                            int lh)
+{
+#pragma unroll
+    for (int d = 0; d < LV; ++d) {
+        const int st = nx >> lh >> (d + 1);  // tw entries between the points of this level's turn
+#pragma unroll
+        for (int q = 0; q < (1 << d); ++q) {
+            const double2 w = __ldg(tw + (lo + (q << lh)) * st);
+#pragma unroll
+            for (int r = q; r < (1 << LV); r += 2 << d)
+                butterfly(z[r], z[r + (1 << d)], w.x, INV ? w.y : -w.y);
         }
     }
-    __syncthreads();
+}
+
+// The transform of a row's nx = 2^lm points by T threads: R0 levels first, then LV at a time
+// (LV divides lm - R0; R0 >= 1), x the row's shared memory.  load(point, q) gives a point (the
+// one q T after the thread's first of a turn); the last pass's go to store(point, value).
+template <int LV, int R0, bool INV, typename Load, typename Store>
+__device__ __forceinline__ void fft_row(double2 *x, const double2 *__restrict__ tw, int nx, int t, int T,
+                                        int lm, Load load, Store store)
+{
+    constexpr int P = 1 << R0, N = 1 << LV, G = N / P;  // points a group, a thread; groups a thread
+    double2 w[4] = {};
+    if (R0 >= 2)
+        w[2] = __ldg(tw + (nx >> 2));
+    if (R0 >= 3) {
+        w[1] = __ldg(tw + (nx >> 3));
+        w[3] = __ldg(tw + 3 * (nx >> 3));
+    }
+    // a group: P points that end up next to each other in bit-reversed order, nx / P apart
+    const int groups = nx >> R0;
+    for (int g0 = t; g0 < groups; g0 += T * G) {
+        double2 z[N];
+#pragma unroll
+        for (int q = 0; q < N; ++q) {
+            const int g = g0 + (q >> R0) * T, r = q & (P - 1);
+            const int rev = R0 == 3 ? ((r & 1) << 2 | (r & 2) | r >> 2) : R0 == 2 ? ((r & 1) << 1 | r >> 1) : r;
+            if (g < groups)
+                z[q] = load(g + rev * groups, (q >> R0) + rev * G);
+        }
+#pragma unroll
+        for (int k = 0; k < G; ++k) {
+            const int g = g0 + k * T;
+            if (g < groups) {
+                first_levels<R0, INV>(z + k * P, w);
+                const int at = lm > R0 ? (int)(__brev((unsigned)g) >> (32 - (lm - R0))) << R0 : 0;
+                const int pl = fft_place(at);
+#pragma unroll
+                for (int r = 0; r < P; ++r) {
+                    if (lm == R0)
+                        store(at + r, z[k * P + r]);
+                    else
+                        x[pl ^ r] = z[k * P + r];
+                }
+            }
+        }
+    }
+    if (lm == R0)
+        return;
+    auto pass = [&](int lh, auto put) {
+        __syncthreads();
+        for (int g = t; g < nx >> LV; g += T) {
+            const int lo = g & ((1 << lh) - 1), at = ((g >> lh) << (lh + LV)) + lo, pl = fft_place(at);
+            double2 z[N];
+#pragma unroll
+            for (int r = 0; r < N; ++r)
+                z[r] = x[pl ^ fft_place(r << lh)];
+            more_levels<LV, INV>(z, tw, nx, lo, lh);
+#pragma unroll
+            for (int r = 0; r < N; ++r)
+                put(at + (r << lh), pl ^ fft_place(r << lh), z[r]);
+        }
+    };
+#pragma unroll 1
+    for (int lh = R0; lh < lm - LV; lh += LV)
+        pass(lh, [&](int, int place, double2 v) { x[place] = v; });
+    pass(lm - LV, [&](int i, int, double2 v) { store(i, v); });
 }
 
 __device__ __forceinline__ double block_sum_fft(double v, double *s_red)
@@ -1619,7 +1757,7 @@ __device__ __forceinline__ double block_sum_fft(double v, double *s_red)
     __syncthreads();
     double t = 0.0;
     if (threadIdx.x == 0)
-        for (int w = 0; w < kFftThreads / 32; ++w)
+        for (int w = 0; w < (int)blockDim.x / 32; ++w)
             t += s_red[w];
     __syncthreads();
     return t;
@@ -1627,47 +1765,108 @@ __device__ __forceinline__ double block_sum_fft(double v, double *s_red)
 
 // forward: b of row j (from the deposits, then cleared, in mode 0; from rho in p.r
 // in mode 1) into p.q, its transform into p.spec; ||b_j||^2 into rpart
-__global__ void __launch_bounds__(kFftThreads) k_fft_rows(Params2D p, int mode)
+template <int LV, int R0>
+__global__ void __launch_bounds__(kFftMaxThreads) k_fft_rows(const __grid_constant__ Params2D p, int mode)
+{
+    constexpr int N = 1 << LV;  // nodes a thread at a time
+    extern __shared__ double2 sx[];
+    __shared__ double s_red[kFftMaxThreads / 32];
+    const int nx = p.nx, ny = p.ny;
+    const int T = fft_row_threads(nx, LV), rows = fft_cta_rows(nx, LV);
+    const int t = threadIdx.x % T, rl = threadIdx.x / T;
+    const int j = 1 + blockIdx.x * rows + rl;
+    const bool act = j < ny;
+    double2 *x = sx + (size_t)rl * nx;
+    const size_t row = (size_t)j * nx;
+    double bb = 0.0;
+    double b[N] = {};  // of N nodes T apart (all of a species' loads in flight at once)
+    if (act)
+        for (int i0 = t; i0 < nx; i0 += T * N) {
+#pragma unroll
+            for (int q = 0; q < N; ++q)
+                b[q] = 0.0;
+            if (mode == 0) {
+                for (int s = 0; s < p.ns; ++s) {
+                    unsigned long long *a = p.acc + (size_t)s * p.nn + row + i0;
+                    const double unit = p.sp[s].rho_unit;
+                    unsigned long long v[N];
+#pragma unroll
+                    for (int q = 0; q < N; ++q)
+                        if (i0 + q * T < nx)
+                            v[q] = a[q * T];
+#pragma unroll
+                    for (int q = 0; q < N; ++q)
+                        if (i0 + q * T < nx) {
+                            b[q] = fma(unit, (double)(long long)v[q], b[q]);
+                            a[q * T] = 0ULL;
+                            // the plate rows' deposits are consumed here too
+                            if (j == 1)
+                                a[q * T - nx] = 0ULL;
+                            if (j == ny - 1)
+                                a[q * T + nx] = 0ULL;
+                        }
+                }
+            } else {
+#pragma unroll
+                for (int q = 0; q < N; ++q)
+                    if (i0 + q * T < nx)
+                        b[q] = p.r[row + i0 + q * T];
+            }
+#pragma unroll
+            for (int q = 0; q < N; ++q)
+                if (i0 + q * T < nx) {
+                    b[q] = p.k2 * b[q];
+                    if (j == 1)
+                        b[q] += p.phi_lo;
+                    if (j == ny - 1)
+                        b[q] += p.phi_hi;
+                    p.q[row + i0 + q * T] = b[q];
+                    bb = fma(b[q], b[q], bb);
+                }
+        }
+    for (int off = min(T, 32) / 2; off; off >>= 1)
+        bb += __shfl_down_sync(0xffffffffu, bb, off, min(T, 32));
+    if (T > 32 && (threadIdx.x & 31) == 0)
+        s_red[threadIdx.x >> 5] = bb;
+    __syncthreads();
+    const double *bq = p.q + row;
+    double2 *out = p.spec + row;
+    const bool one = T * N >= nx;  // the row is in registers
+    fft_row<LV, R0, false>(
+        x, p.tw, nx, t, T, p.log2nx,
+        [&](int i, int q) { return make_double2(one ? b[q] : act ? bq[i] : 0.0, 0.0); },
+        [&](int i, double2 v) {
+            if (act)
+                out[i] = v;
+        });
+    if (t == 0 && act) {
+        if (T > 32)
+            for (int w = 1; w < T / 32; ++w)
+                bb += s_red[w];
+        p.rpart[2 * j + 1] = bb;
+    }
+}
+
+// inverse: phi of row j from its coefficients
+template <int LV, int R0>
+__global__ void __launch_bounds__(kFftMaxThreads) k_ifft_rows(const __grid_constant__ Params2D p)
 {
     extern __shared__ double2 sx[];
-    __shared__ double s_red[kFftThreads / 32];
-    const int nx = p.nx, ny = p.ny, j = blockIdx.x + 1;
-    const int shift = 32 - p.log2nx;
-    double bb = 0.0;
-    for (int i = threadIdx.x; i < nx; i += kFftThreads) {
-        const int idx = j * nx + i;
-        double rho = 0.0;
-        if (mode == 0) {
-            for (int s = 0; s < p.ns; ++s) {
-                unsigned long long *a = p.acc + (size_t)s * p.nn + idx;
-                rho = fma(p.sp[s].rho_unit, (double)(long long)*a, rho);
-                *a = 0ULL;
-            }
-            // the plate rows' deposits are consumed here too
-            if (j == 1)
-                for (int s = 0; s < p.ns; ++s)
-                    p.acc[(size_t)s * p.nn + i] = 0ULL;
-            if (j == ny - 1)
-                for (int s = 0; s < p.ns; ++s)
-                    p.acc[(size_t)s * p.nn + (size_t)ny * nx + i] = 0ULL;
-        } else {
-            rho = p.r[idx];
-        }
-        double b = p.k2 * rho;
-        if (j == 1)
-            b += p.phi_lo;
-        if (j == ny - 1)
-            b += p.phi_hi;
-        p.q[idx] = b;
-        bb = fma(b, b, bb);
-        sx[__brev((unsigned)i) >> shift] = make_double2(b, 0.0);
-    }
-    const double bbs = block_sum_fft(bb, s_red);
-    if (threadIdx.x == 0)
-        p.rpart[2 * j + 1] = bbs;
-    fft_smem(sx, p.tw, nx, -1.0);
-    for (int k = threadIdx.x; k < nx; k += kFftThreads)
-        p.spec[(size_t)j * nx + k] = sx[k];
+    const int nx = p.nx;
+    const int T = fft_row_threads(nx, LV), rows = fft_cta_rows(nx, LV);
+    const int t = threadIdx.x % T, rl = threadIdx.x / T;
+    const int j = 1 + blockIdx.x * rows + rl;
+    const bool act = j < p.ny;
+    const double inv = 1.0 / nx;
+    const double2 *in = p.spec + (size_t)j * nx;
+    double *phi = p.phi + (size_t)j * nx;
+    fft_row<LV, R0, true>(
+        sx + (size_t)rl * nx, p.tw, nx, t, T, p.log2nx,
+        [&](int i, int) { return act ? in[i] : make_double2(0.0, 0.0); },
+        [&](int i, double2 v) {
+            if (act)
+                phi[i] = v.x * inv;
+        });
 }
 
 // Thomas per mode k: forward u'_j = (b^_j + u'_{j-1}) / m_j, back u_j = u'_j + u_{j+1} / m_j
@@ -1676,158 +1875,238 @@ __global__ void __launch_bounds__(kFftThreads) k_fft_rows(Params2D p, int mode)
 // from a zero start (x~), then the value entering each segment by a short sequential
 // pass over the segments' ends, then x = x~ + P x_in with P the product of the
 // segment's multipliers up to the row (tabulated: seg_f forward, seg_b backward).
-// A CTA takes kTriModes modes (consecutive k: coalesced rows) times kTriSegs segments.
-constexpr int kTriModes = 8;
+// A CTA takes kTriModes modes (consecutive: 64 bytes a row) times kTriSegs segments.  What a
+// step of a chain costs is FP64 latency (110 cycles on an idle pipe), if its operands are
+// there: a batch of rows is loaded at once, the segments' ends and products are gathered
+// before the sequential pass, and between the passes the values stay in shared memory
+// where they fit (kShared; ny up to some 3,500), else in the coefficients' place.
+constexpr int kTriModes = 4;
 constexpr int kTriSegs = 32;
+constexpr int kTriBatch = 8;
 
 __host__ __device__ __forceinline__ int tri_seg_len(int ny)
 {
     return (ny - 1 + kTriSegs - 1) / kTriSegs;
 }
 
-__global__ void __launch_bounds__(kTriModes * kTriSegs) k_tridiag_modes(Params2D p)
+// shared memory of kShared: an odd number of rows a segment, so that the segments that a
+// warp's threads work on lie in different banks
+size_t tri_smem_bytes(int ny)
 {
-    __shared__ double2 s_end[kTriSegs][kTriModes], s_in[kTriSegs][kTriModes];
+    return sizeof(double2) * kTriModes * kTriSegs * (size_t)(tri_seg_len(ny) | 1);
+}
+
+struct TriEnds {
+    double2 end[kTriSegs][kTriModes], in[kTriSegs][kTriModes];  // values leaving (from zero), entering
+    double prod[kTriSegs][kTriModes];                           // the product of a segment's multipliers
+};
+
+// the value entering each segment, in order (or from the last): a thread per mode
+__device__ __forceinline__ void tri_chain(TriEnds &e, int kk, int used, bool back)
+{
+    double2 c = make_double2(0.0, 0.0);
+#pragma unroll 8
+    for (int i = 0; i < used; ++i) {
+        const int t = back ? used - 1 - i : i;
+        e.in[t][kk] = c;
+        const double f = e.prod[t][kk];
+        const double2 v = e.end[t][kk];
+        c = make_double2(fma(f, c.x, v.x), fma(f, c.y, v.y));
+    }
+}
+
+template <bool kShared>
+__global__ void __launch_bounds__(kTriModes * kTriSegs) k_tridiag_modes(const __grid_constant__ Params2D p)
+{
+    extern __shared__ double2 s_x[];
+    __shared__ TriEnds e;
     const int nx = p.nx, ny = p.ny;
     const int kk = threadIdx.x % kTriModes, sg = threadIdx.x / kTriModes;
     const int k = blockIdx.x * kTriModes + kk;
-    const bool act = k < nx;
-    const int L = tri_seg_len(ny);
-    const int j0 = 1 + sg * L, j1 = min(ny, j0 + L);  // this segment's rows [j0, j1)
-    double2 *__restrict__ spec = p.spec;
-    const double *__restrict__ invm = p.inv_m;
-    const double *__restrict__ pf = p.seg_f;
-    const double *__restrict__ pb = p.seg_b;
+    const int L = tri_seg_len(ny), used = (ny - 1 + L - 1) / L;  // segments with rows
+    // this segment's rows [j0, j1) (64 bits: the last segments may start far past ny)
+    const int j0 = (int)min((long long)ny, 1 + (long long)sg * L);
+    const int j1 = k < nx ? (int)min((long long)ny, (long long)j0 + L) : j0;
+    const size_t first = (size_t)j0 * nx + k;
+    double2 *__restrict__ spec = p.spec + first;
+    const double *__restrict__ invm = p.inv_m + first;
+    const double *__restrict__ pf = p.seg_f + first;
+    const double *__restrict__ pb = p.seg_b + first;
+    double2 *xv = kShared ? s_x + (size_t)sg * (L | 1) * kTriModes + kk : spec;
+    const size_t xs = kShared ? kTriModes : nx;  // from row to row
+    const int rows = j1 - j0;
     // 1. forward, from zero
     double2 x = make_double2(0.0, 0.0);
-    if (act)
-        for (int j = j0; j < j1; ++j) {
-            const size_t o = (size_t)j * nx + k;
-            const double2 v = spec[o];
-            const double m = __ldg(invm + o);
-            x = make_double2((v.x + x.x) * m, (v.y + x.y) * m);
-            spec[o] = x;
-        }
-    s_end[sg][kk] = x;
-    __syncthreads();
-    // 2. the forward value entering each segment (a thread per mode)
-    if (sg == 0 && act) {
-        double2 c = make_double2(0.0, 0.0);
-        for (int t = 0; t < kTriSegs; ++t) {
-            s_in[t][kk] = c;
-            const int e = min(ny, 1 + (t + 1) * L) - 1;  // the segment's last row
-            if (1 + t * L <= e) {
-                const double f = __ldg(pf + (size_t)e * nx + k);
-                c = make_double2(fma(f, c.x, s_end[t][kk].x), fma(f, c.y, s_end[t][kk].y));
+#pragma unroll 1
+    for (int b = 0; b < rows; b += kTriBatch) {
+        double2 v[kTriBatch];
+        double m[kTriBatch];
+#pragma unroll
+        for (int i = 0; i < kTriBatch; ++i)
+            if (b + i < rows) {
+                v[i] = spec[(size_t)(b + i) * nx];
+                m[i] = __ldg(invm + (size_t)(b + i) * nx);
             }
-        }
+#pragma unroll
+        for (int i = 0; i < kTriBatch; ++i)
+            if (b + i < rows) {
+                x = make_double2((v[i].x + x.x) * m[i], (v[i].y + x.y) * m[i]);
+                xv[(b + i) * xs] = x;
+            }
     }
+    e.end[sg][kk] = x;
+    e.prod[sg][kk] = rows > 0 ? __ldg(pf + (size_t)(rows - 1) * nx) : 0.0;
+    __syncthreads();
+    // 2. the forward value entering each segment
+    if (sg == 0)
+        tri_chain(e, kk, used, false);
     __syncthreads();
     // 3. the forward values completed, then the backward recurrence from zero, top down
-    const double2 cf = s_in[sg][kk];
+    const double2 cf = e.in[sg][kk];
     double2 u = make_double2(0.0, 0.0);
-    if (act)
-        for (int j = j1 - 1; j >= j0; --j) {
-            const size_t o = (size_t)j * nx + k;
-            const double f = __ldg(pf + o);
-            const double2 v = spec[o];
-            const double2 d = make_double2(fma(f, cf.x, v.x), fma(f, cf.y, v.y));
-            const double m = __ldg(invm + o);
-            u = make_double2(fma(u.x, m, d.x), fma(u.y, m, d.y));
-            spec[o] = u;
-        }
-    __syncthreads();  // every thread has read s_in
-    s_end[sg][kk] = u;
+#pragma unroll 1
+    for (int b = rows - 1; b >= 0; b -= kTriBatch) {
+        double2 v[kTriBatch];
+        double m[kTriBatch], f[kTriBatch];
+#pragma unroll
+        for (int i = 0; i < kTriBatch; ++i)
+            if (b - i >= 0) {
+                v[i] = xv[(b - i) * xs];
+                m[i] = __ldg(invm + (size_t)(b - i) * nx);
+                f[i] = __ldg(pf + (size_t)(b - i) * nx);
+            }
+#pragma unroll
+        for (int i = 0; i < kTriBatch; ++i)
+            if (b - i >= 0) {
+                u = make_double2(fma(u.x, m[i], fma(f[i], cf.x, v[i].x)),
+                                 fma(u.y, m[i], fma(f[i], cf.y, v[i].y)));
+                xv[(b - i) * xs] = u;
+            }
+    }
+    __syncthreads();  // every thread has read its value of pass 2
+    e.end[sg][kk] = u;
+    e.prod[sg][kk] = rows > 0 ? __ldg(pb) : 0.0;
     __syncthreads();
     // 4. the backward value entering each segment from above
-    if (sg == 0 && act) {
-        double2 c = make_double2(0.0, 0.0);
-        for (int t = kTriSegs - 1; t >= 0; --t) {
-            s_in[t][kk] = c;
-            const int b0 = 1 + t * L;  // the segment's first row
-            if (b0 <= min(ny, b0 + L) - 1) {
-                const double g = __ldg(pb + (size_t)b0 * nx + k);
-                c = make_double2(fma(g, c.x, s_end[t][kk].x), fma(g, c.y, s_end[t][kk].y));
-            }
-        }
-    }
+    if (sg == 0)
+        tri_chain(e, kk, used, true);
     __syncthreads();
     // 5. the backward values completed
-    const double2 cb = s_in[sg][kk];
-    if (act)
-        for (int j = j0; j < j1; ++j) {
-            const size_t o = (size_t)j * nx + k;
-            const double g = __ldg(pb + o);
-            const double2 w = spec[o];
-            spec[o] = make_double2(fma(g, cb.x, w.x), fma(g, cb.y, w.y));
-        }
+    const double2 cb = e.in[sg][kk];
+#pragma unroll 1
+    for (int b = 0; b < rows; b += kTriBatch) {
+        double2 v[kTriBatch];
+        double g[kTriBatch];
+#pragma unroll
+        for (int i = 0; i < kTriBatch; ++i)
+            if (b + i < rows) {
+                v[i] = xv[(b + i) * xs];
+                g[i] = __ldg(pb + (size_t)(b + i) * nx);
+            }
+#pragma unroll
+        for (int i = 0; i < kTriBatch; ++i)
+            if (b + i < rows)
+                spec[(size_t)(b + i) * nx] =
+                    make_double2(fma(g[i], cb.x, v[i].x), fma(g[i], cb.y, v[i].y));
+    }
 }
 
-// inverse: phi of row j from its coefficients
-__global__ void __launch_bounds__(kFftThreads) k_ifft_rows(Params2D p)
+// E on every node (mode 0) and the true residual r = b - A phi per row, a row per CTA, two
+// nodes a thread; the last CTA adds the rows' sums in a fixed order (contiguous runs of
+// rows per thread, then a fixed tree: the same result every run) and keeps the books.
+__global__ void __launch_bounds__(kFinishThreads) k_fft_finish(const __grid_constant__ Params2D p, int mode)
 {
-    extern __shared__ double2 sx[];
-    const int nx = p.nx, j = blockIdx.x + 1;
-    const int shift = 32 - p.log2nx;
-    for (int k = threadIdx.x; k < nx; k += kFftThreads)
-        sx[__brev((unsigned)k) >> shift] = p.spec[(size_t)j * nx + k];
-    fft_smem(sx, p.tw, nx, 1.0);
-    const double inv = 1.0 / nx;
-    for (int i = threadIdx.x; i < nx; i += kFftThreads)
-        p.phi[(size_t)j * nx + i] = sx[i].x * inv;
-}
-
-// E on every node (mode 0) and the true residual r = b - A phi per row
-__global__ void __launch_bounds__(kFftThreads) k_fft_finish(Params2D p, int mode)
-{
-    __shared__ double s_red[kFftThreads / 32];
+    __shared__ double s_red[kFinishThreads / 32];
+    __shared__ bool s_last;
     const int nx = p.nx, ny = p.ny, j = blockIdx.x;  // rows 0..ny
+    const double h = p.half_dx;
     double rr = 0.0;
-    for (int i = threadIdx.x; i < nx; i += kFftThreads) {
-        const int idx = j * nx + i;
-        if (mode == 0)
-            store_E(p, idx);
+    const double *__restrict__ f = p.phi + (size_t)j * nx;
+    for (int i = 2 * threadIdx.x; i < nx; i += 2 * kFinishThreads) {
+        const double2 c = *reinterpret_cast<const double2 *>(f + i);
+        const double l = f[i == 0 ? nx - 1 : i - 1], r = f[i + 2 == nx ? 0 : i + 2];
+        double2 up = make_double2(0.0, 0.0), dn = up;
+        if (j < ny)
+            up = *reinterpret_cast<const double2 *>(f + nx + i);
+        if (j > 0)
+            dn = *reinterpret_cast<const double2 *>(f - nx + i);
+        if (mode == 0) {
+            double2 ey;
+            if (j == 0)
+                ey = make_double2(-(up.x - c.x) / p.dx, -(up.y - c.y) / p.dx);
+            else if (j == ny)
+                ey = make_double2(-(c.x - dn.x) / p.dx, -(c.y - dn.y) / p.dx);
+            else
+                ey = make_double2(-(up.x - dn.x) * h, -(up.y - dn.y) * h);
+            *reinterpret_cast<float4 *>(p.E + (size_t)j * nx + i) =
+                make_float4((float)(-(c.y - l) * h), (float)ey.x, (float)(-(r - c.x) * h), (float)ey.y);
+        }
         if (j >= 1 && j < ny) {
-            const int ip = (i + 1 == nx) ? idx + 1 - nx : idx + 1;
-            const int im = (i == 0) ? idx - 1 + nx : idx - 1;
-            const double *f = p.phi;
-            double ap = 4.0 * f[idx] - (f[ip] + f[im]);
-            if (j > 1)
-                ap -= f[idx - nx];
-            if (j < ny - 1)
-                ap -= f[idx + nx];
-            const double r = p.q[idx] - ap;
-            rr = fma(r, r, rr);
+            const double2 q = *reinterpret_cast<const double2 *>(p.q + (size_t)j * nx + i);
+            double a0 = 4.0 * c.x - (c.y + l), a1 = 4.0 * c.y - (r + c.x);
+            if (j > 1) {
+                a0 -= dn.x;
+                a1 -= dn.y;
+            }
+            if (j < ny - 1) {
+                a0 -= up.x;
+                a1 -= up.y;
+            }
+            const double r0 = q.x - a0, r1 = q.y - a1;
+            rr = fma(r0, r0, rr);
+            rr = fma(r1, r1, rr);
         }
     }
     const double rrs = block_sum_fft(rr, s_red);
-    if (threadIdx.x == 0)
+    if (threadIdx.x == 0) {
         p.rpart[2 * j] = (j >= 1 && j < ny) ? rrs : 0.0;
-}
-
-// the per-row sums added in a fixed order (contiguous runs of rows per thread, then
-// a fixed tree: the same result every run) and the bookkeeping of a solve
-__global__ void __launch_bounds__(kFftThreads) k_fft_report(Params2D p)
-{
-    __shared__ double s_red[kFftThreads / 32];
-    const int rows = p.ny - 1, per = (rows + kFftThreads - 1) / kFftThreads;
+        __threadfence();
+        const unsigned n = atomicAdd(p.finished, 1u);
+        s_last = n == gridDim.x - 1;
+    }
+    __syncthreads();
+    if (!s_last)
+        return;
+    __threadfence();
+    const int rows = ny - 1, per = (rows + kFinishThreads - 1) / kFinishThreads;
     double r = 0.0, b = 0.0;
     for (int q = 0; q < per; ++q) {
-        const int j = 1 + threadIdx.x * per + q;
-        if (j < p.ny) {
-            r += p.rpart[2 * j];
-            b += p.rpart[2 * j + 1];
+        const int m = 1 + threadIdx.x * per + q;
+        if (m < ny) {
+            r += __ldcg(p.rpart + 2 * m);
+            b += __ldcg(p.rpart + 2 * m + 1);
         }
     }
     const double R = block_sum_fft(r, s_red);
     const double B = block_sum_fft(b, s_red);
     if (threadIdx.x != 0)
         return;
+    *p.finished = 0u;
     State2D *st = p.st;
     st->cg_iters = 0;
     st->cg_res = B > 0.0 ? sqrt(R / B) : 0.0;
     if (B > 0.0 && R > p.rtol2 * B)
         atomicCAS(&st->error, 0, SLPIC_ERR_NOCONVERGE);
+}
+
+// the instantiation for a grid
+typedef void (*FftKernel)(Params2D, int);
+typedef void (*IfftKernel)(Params2D);
+
+FftKernel fft_kernel(const Params2D &p)
+{
+    if (fft_levels(p.nx, p.ny) == 1)
+        return k_fft_rows<1, 1>;
+    const int r = p.log2nx % 3;
+    return r == 1 ? k_fft_rows<3, 1> : r == 2 ? k_fft_rows<3, 2> : k_fft_rows<3, 3>;
+}
+
+IfftKernel ifft_kernel(const Params2D &p)
+{
+    if (fft_levels(p.nx, p.ny) == 1)
+        return k_ifft_rows<1, 1>;
+    const int r = p.log2nx % 3;
+    return r == 1 ? k_ifft_rows<3, 1> : r == 2 ? k_ifft_rows<3, 2> : k_ifft_rows<3, 3>;
 }
 
 // ---- counting sort of the particles by cell ------------------------------------------
@@ -2076,6 +2355,7 @@ struct slpic2d_sim {
     int ctas = 1;     // particle-kernel CTAs per species
     int tile_ctas = 0;  // k_particles2d_tiles CTAs per species (0: not resident)
     int hard_ctas = 1;  // k_hard2d: all resident
+    size_t tri_smem = 0;  // k_tridiag_modes' shared memory (0: the values do not fit)
     int small_ctas = 1; // k_inject2d: 2 CTAs of 256 threads per SM
     bool prepared = false;
     bool timing = false;               // record events around the kernels of each step
@@ -2229,12 +2509,16 @@ static int launch_solve(slpic2d_t *h, int mode)
     if (h->p.solver != SLPIC2D_SOLVER_FFT)
         return launch_cg(h, mode);
     const Params2D &p = h->p;
-    const size_t smem = (size_t)16 * p.nx;
-    k_fft_rows<<<p.ny - 1, kFftThreads, smem, h->stream>>>(p, mode);
-    k_tridiag_modes<<<(p.nx + kTriModes - 1) / kTriModes, kTriModes * kTriSegs, 0, h->stream>>>(p);
-    k_ifft_rows<<<p.ny - 1, kFftThreads, smem, h->stream>>>(p);
-    k_fft_finish<<<p.ny + 1, kFftThreads, 0, h->stream>>>(p, mode);
-    k_fft_report<<<1, kFftThreads, 0, h->stream>>>(p);
+    const int lv = fft_levels(p.nx, p.ny), rows = fft_cta_rows(p.nx, lv), threads = rows * fft_row_threads(p.nx, lv);
+    const int ctas = (p.ny - 1 + rows - 1) / rows, tri = (p.nx + kTriModes - 1) / kTriModes;
+    const size_t smem = (size_t)16 * rows * p.nx;
+    fft_kernel(p)<<<ctas, threads, smem, h->stream>>>(p, mode);
+    if (h->tri_smem)
+        k_tridiag_modes<true><<<tri, kTriModes * kTriSegs, h->tri_smem, h->stream>>>(p);
+    else
+        k_tridiag_modes<false><<<tri, kTriModes * kTriSegs, 0, h->stream>>>(p);
+    ifft_kernel(p)<<<ctas, threads, smem, h->stream>>>(p);
+    k_fft_finish<<<p.ny + 1, kFinishThreads, 0, h->stream>>>(p, mode);
     CK2(h, cudaGetLastError());
     return SLPIC_OK;
 }
@@ -2321,6 +2605,7 @@ extern "C" int slpic2d_create(const slpic2d_config *c, slpic2d_t **out)
     p.dx = c->dx;
     p.dt64 = c->dt;
     p.k2 = c->dx * c->dx / c->eps0;
+    p.half_dx = 0.5 / c->dx;
     p.phi_lo = c->phi_lo;
     p.phi_hi = c->phi_hi;
     p.rtol2 = c->cg_rtol * c->cg_rtol;
@@ -2395,54 +2680,66 @@ extern "C" int slpic2d_create(const slpic2d_config *c, slpic2d_t **out)
         p.log2nx = 0;
         while ((1 << p.log2nx) < p.nx)
             ++p.log2nx;
-        if (!alloc((void **)&p.tw, sizeof(double2) * std::max(1, p.nx / 2)) ||
+        if (!alloc((void **)&p.tw, sizeof(double2) * (p.nx / 2)) ||
             !alloc((void **)&p.spec, sizeof(double2) * nn) ||
             !alloc((void **)&p.inv_m, sizeof(double) * nn) ||
             !alloc((void **)&p.seg_f, sizeof(double) * nn) ||
             !alloc((void **)&p.seg_b, sizeof(double) * nn) ||
-            !alloc((void **)&p.rpart, sizeof(double) * 2 * (p.ny + 1)))
+            !alloc((void **)&p.rpart, sizeof(double) * 2 * (p.ny + 1)) ||
+            !alloc((void **)&p.finished, sizeof(unsigned)))
             return bail(SLPIC_ERR_OOM, "device allocation failed");
         const double two_pi = 6.283185307179586;
-        std::vector<double2> tw((size_t)std::max(1, p.nx / 2));
+        std::vector<double2> tw((size_t)p.nx / 2);
         for (int m = 0; m < p.nx / 2; ++m)
             tw[m] = make_double2(std::cos(two_pi * m / p.nx), std::sin(two_pi * m / p.nx));
-        std::vector<double> inv_m(nn, 0.0);
+        // the multipliers and their products within each segment of rows (k_tridiag_modes)
+        std::vector<double> tables(3 * nn, 0.0);
+        double *inv_m = tables.data(), *seg_f = inv_m + nn, *seg_b = seg_f + nn;
+        const int L = tri_seg_len(p.ny);
         for (int k = 0; k < p.nx; ++k) {
+            const auto at = [&](int j) { return (size_t)j * p.nx + k; };
             const double a = 4.0 - 2.0 * std::cos(two_pi * k / p.nx);
             double prev = 0.0;  // 1/m_{j-1}
             for (int j = 1; j < p.ny; ++j) {
                 prev = 1.0 / (a - prev);
-                inv_m[(size_t)j * p.nx + k] = prev;
+                inv_m[at(j)] = prev;
             }
-        }
-        // products of the multipliers within each segment of rows (k_tridiag_modes)
-        std::vector<double> seg_f(nn, 0.0), seg_b(nn, 0.0);
-        const int L = tri_seg_len(p.ny);
-        for (int k = 0; k < p.nx; ++k)
             for (int j0 = 1; j0 < p.ny; j0 += L) {
                 const int j1 = std::min(p.ny, j0 + L);
                 double f = 1.0, g = 1.0;
                 for (int j = j0; j < j1; ++j) {
-                    f *= inv_m[(size_t)j * p.nx + k];
-                    seg_f[(size_t)j * p.nx + k] = f;
+                    f *= inv_m[at(j)];
+                    seg_f[at(j)] = f;
                 }
                 for (int j = j1 - 1; j >= j0; --j) {
-                    g *= inv_m[(size_t)j * p.nx + k];
-                    seg_b[(size_t)j * p.nx + k] = g;
+                    g *= inv_m[at(j)];
+                    seg_b[at(j)] = g;
                 }
             }
+        }
         cudaError_t e2 = cudaMemcpy(p.tw, tw.data(), sizeof(double2) * tw.size(), cudaMemcpyHostToDevice);
         if (e2 == cudaSuccess)
-            e2 = cudaMemcpy(p.inv_m, inv_m.data(), sizeof(double) * nn, cudaMemcpyHostToDevice);
+            e2 = cudaMemcpy(p.inv_m, inv_m, sizeof(double) * nn, cudaMemcpyHostToDevice);
         if (e2 == cudaSuccess)
-            e2 = cudaMemcpy(p.seg_f, seg_f.data(), sizeof(double) * nn, cudaMemcpyHostToDevice);
+            e2 = cudaMemcpy(p.seg_f, seg_f, sizeof(double) * nn, cudaMemcpyHostToDevice);
         if (e2 == cudaSuccess)
-            e2 = cudaMemcpy(p.seg_b, seg_b.data(), sizeof(double) * nn, cudaMemcpyHostToDevice);
-        const int smem = 16 * p.nx;
+            e2 = cudaMemcpy(p.seg_b, seg_b, sizeof(double) * nn, cudaMemcpyHostToDevice);
+        if (e2 == cudaSuccess)
+            e2 = cudaMemset(p.finished, 0, sizeof(unsigned));
+        const size_t tri = tri_smem_bytes(p.ny);
+        int most = 0;
+        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+        if (e2 == cudaSuccess && tri + sizeof(TriEnds) <= (size_t)most) {
+            h->tri_smem = tri;
+            if (tri > 32 * 1024)
+                e2 = cudaFuncSetAttribute(k_tridiag_modes<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          (int)tri);
+        }
+        const int smem = 16 * p.nx * fft_cta_rows(p.nx, fft_levels(p.nx, p.ny));
         if (e2 == cudaSuccess && smem > 48 * 1024)
-            e2 = cudaFuncSetAttribute(k_fft_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            e2 = cudaFuncSetAttribute(fft_kernel(p), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e2 == cudaSuccess && smem > 48 * 1024)
-            e2 = cudaFuncSetAttribute(k_ifft_rows, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            e2 = cudaFuncSetAttribute(ifft_kernel(p), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
         if (e2 != cudaSuccess)
             return bail(SLPIC_ERR_CUDA, cudaGetErrorString(e2));
     }
