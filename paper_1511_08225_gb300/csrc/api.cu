@@ -87,8 +87,8 @@ struct slpic_sim {
 
     std::vector<slpic_sim *> members;
     StepParams *d_params = nullptr;  // [members] on the device
-    int4 *d_work = nullptr;          // particle-kernel work items
-    int n_work = 0, max_nn = 0, max_ns = 0, batch_hard_ctas = 4;
+    BatchWork work[2];               // the particle kernels' work items: in place, compacting
+    int max_nn = 0, max_ns = 0, batch_hard_ctas = 4;
 
     std::string err;
 };
@@ -472,7 +472,10 @@ extern "C" int slpic_destroy(slpic_t *h)
     for (slpic_t *m : h->members)
         slpic_destroy(m);
     cudaFree(h->d_params);
-    cudaFree(h->d_work);
+    for (BatchWork &w : h->work) {
+        cudaFree(w.items);
+        cudaFree(w.first);
+    }
     free_all(h);
     delete h;
     return SLPIC_OK;
@@ -1475,23 +1478,25 @@ extern "C" int slpic_create_batch(const slpic_config *cfgs, int m, slpic_t **out
     if (cudaMalloc(&h->d_params, sizeof(StepParams) * m) != cudaSuccess)
         return bail(SLPIC_ERR_OOM, "device allocation failed");
     int occ = 0, occ_c = 0;
-    if (configure_batch_kernels(h->max_nn, &occ, &occ_c) != cudaSuccess || occ < 1 || occ_c < 1)
+    if (configure_batch_kernels(h->max_nn, &occ, &occ_c, &h->tma_stages) != cudaSuccess || occ < 1 || occ_c < 1)
         return bail(SLPIC_ERR_INVALID, "batched particle kernel cannot be resident");
     h->ctas = occ;     // resident batched CTAs per SM (work-table sizing)
     h->ctas_c = occ_c;
-    // the iterative-push kernel: the single simulation's whole-GPU grid, shared out
-    h->batch_hard_ctas = std::max(4, h->num_sms * 8 / m);
+    h->batch_hard_ctas = h->num_sms * 4;  // the iterative-push kernel: all resident
     *out = h;
     return SLPIC_OK;
 }
 
-// Work items of the batched particle kernels: every (instance, species) gets CTAs
-// in proportion to its particles (at least one), about `waves` full waves of the GPU.
+// Work items of the batched particle kernels: the (instance, species) pairs' particles laid
+// end to end and cut into as many equal parts as there are CTAs (`waves` full waves of the
+// GPU, fewer if the parts would be smaller than `min_share`, but at least one CTA a pair).
 static int batch_tables(slpic_t *h)
 {
-    std::vector<long long> n;
+    std::vector<int2> pair;           // instance, species
+    std::vector<long long> n, start;  // particles, and those of the pairs before
     long long total = 0;
-    for (slpic_t *m : h->members) {
+    for (int i = 0; i < (int)h->members.size(); ++i) {
+        slpic_t *m = h->members[i];
         DevState st;
         int rc = read_state(m, &st);
         if (rc) {
@@ -1500,29 +1505,44 @@ static int batch_tables(slpic_t *h)
         }
         const int P = (int)(m->step & 1);
         for (int s = 0; s < m->ns; ++s) {
-            n.push_back((long long)st.count[s][P]);
-            total += (long long)st.count[s][P];
+            pair.push_back(make_int2(i, s));
+            n.push_back((long long)st.count[s][P] + 1);  // (one more: none is without weight)
+            start.push_back(total);
+            total += n.back();
         }
     }
-    const int waves = h->batch_waves;
-    const long long budget = (long long)h->num_sms * std::min(h->ctas, h->ctas_c) * waves;
-    std::vector<int4> work;
-    size_t k = 0;
-    for (int i = 0; i < (int)h->members.size(); ++i) {
-        for (int s = 0; s < h->members[i]->ns; ++s, ++k) {
-            long long c = total > 0 ? (n[k] * budget + total - 1) / total : 1;
-            // a share large enough to amortise the per-CTA grid staging
-            const long long per = std::max(1LL, n[k] / h->batch_min_share);
-            c = std::max(1LL, std::min(c, per));
-            for (int j = 0; j < (int)c; ++j)
-                work.push_back(make_int4(i, s, j, (int)c));
+    for (int compact = 0; compact < 2; ++compact) {
+        const long long places = (long long)h->num_sms * (compact ? h->ctas_c : h->ctas) * h->batch_waves;
+        const long long fewest = std::max<long long>(total / h->batch_min_share, (long long)pair.size());
+        const int ctas = (int)std::min(places, fewest);
+        std::vector<int4> items;
+        std::vector<int> first;
+        size_t k = 0;
+        for (int b = 0; b < ctas; ++b) {
+            first.push_back((int)items.size());
+            const long long hi = total * (b + 1) / ctas;
+            for (; k < pair.size() && start[k] < hi; ++k) {
+                const long long lo = std::max(total * b / ctas, start[k]);
+                const bool ends = start[k] + n[k] <= hi;
+                const int f0 = (int)((double)(lo - start[k]) / (double)n[k] * kBatchParts);
+                const int f1 = ends ? kBatchParts : (int)((double)(hi - start[k]) / (double)n[k] * kBatchParts);
+                if (f1 > f0)
+                    items.push_back(make_int4(pair[k].x, pair[k].y, f0, f1));
+                if (!ends)
+                    break;  // the next CTA goes on with it
+            }
         }
+        first.push_back((int)items.size());
+        BatchWork &w = h->work[compact];
+        cudaFree(w.items);
+        cudaFree(w.first);
+        w = BatchWork();
+        CK(h, cudaMalloc(&w.items, sizeof(int4) * std::max<size_t>(1, items.size())));
+        CK(h, cudaMalloc(&w.first, sizeof(int) * first.size()));
+        CK(h, cudaMemcpy(w.items, items.data(), sizeof(int4) * items.size(), cudaMemcpyHostToDevice));
+        CK(h, cudaMemcpy(w.first, first.data(), sizeof(int) * first.size(), cudaMemcpyHostToDevice));
+        w.ctas = ctas;
     }
-    cudaFree(h->d_work);
-    h->d_work = nullptr;
-    CK(h, cudaMalloc(&h->d_work, sizeof(int4) * work.size()));
-    CK(h, cudaMemcpy(h->d_work, work.data(), sizeof(int4) * work.size(), cudaMemcpyHostToDevice));
-    h->n_work = (int)work.size();
     return SLPIC_OK;
 }
 
@@ -1559,7 +1579,7 @@ static int batch_capture(slpic_t *h, long long first_step, int nsteps, cudaGraph
     CK(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
     for (int k = 0; k < nsteps; ++k) {
         const bool compact = (first_step + k) % h->compact_every == h->compact_every - 1;
-        launch_particles_batch(h->d_params, h->d_work, h->n_work, h->max_nn, compact,
+        launch_particles_batch(h->d_params, h->work[compact], h->max_nn, compact, h->tma_stages,
                                h->cap_stream);
         launch_hard_batch(h->d_params, m, h->batch_hard_ctas, compact, h->cap_stream);
         launch_field_batch(h->d_params, m, h->max_nn, h->max_ns, compact ? 2 : 1, h->cap_stream);

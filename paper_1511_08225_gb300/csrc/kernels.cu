@@ -153,9 +153,10 @@ __device__ __forceinline__ void list_hard(bool hard, long long i, int c, const f
 }
 
 // Bodies of the kernels take the parameters by reference (kernel parameter space
-// for one simulation, shared memory for a batch) and the CTA's share of the work.
+// for one simulation, shared memory for a batch) and the CTA's share of the work: the
+// species' tiles from f0 to f1 of `parts`.
 template <bool kProf, int kKind = kAny, int kPer = kAny>
-__device__ __forceinline__ void particles_compact(const StepParams &p, int s, int cta, int nctas)
+__device__ __forceinline__ void particles_compact(const StepParams &p, int s, int f0, int f1, int parts)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned *s_lo = reinterpret_cast<unsigned *>(smem);  // [nn] deposit, low words
@@ -187,8 +188,8 @@ __device__ __forceinline__ void particles_compact(const StepParams &p, int s, in
 
     DepositSplit32 dep{s_lo, s_hi};
     const long long ntiles = (n + kPT - 1) / kPT;
-    const long long t0 = ntiles * cta / nctas;
-    const long long t1 = ntiles * (cta + 1) / nctas;
+    const long long t0 = ntiles * f0 / parts;
+    const long long t1 = ntiles * f1 / parts;
 
     for (long long t = t0; t < t1; ++t) {
         const long long base = t * kPT;
@@ -247,7 +248,7 @@ constexpr int kWT = 32 * kWI;    // particles per warp-tile
 size_t particle_inplace_smem_bytes(int nn) { return (size_t)nn * 3 * sizeof(unsigned); }
 
 template <bool kProf, int kKind = kAny, int kPer = kAny>
-__device__ __forceinline__ void particles_inplace(const StepParams &p, int s, int cta, int nctas)
+__device__ __forceinline__ void particles_inplace(const StepParams &p, int s, int f0, int f1, int parts)
 {
     extern __shared__ __align__(16) unsigned char smem[];
     unsigned *s_lo = reinterpret_cast<unsigned *>(smem);  // [nn] deposit, low words
@@ -281,8 +282,8 @@ __device__ __forceinline__ void particles_inplace(const StepParams &p, int s, in
     // warp-tiles of kWT consecutive particles: the CTA owns a contiguous range of
     // them and its warps take every kNW-th
     const long long nwt = (n + kWT - 1) / kWT;
-    const long long w0 = nwt * cta / nctas;
-    const long long w1 = nwt * (cta + 1) / nctas;
+    const long long w0 = nwt * f0 / parts;
+    const long long w1 = nwt * f1 / parts;
     for (long long t = w0 + warp; t < w1; t += kNW) {
         const long long base = t * kWT;
         int c[kWI];
@@ -299,6 +300,15 @@ __device__ __forceinline__ void particles_inplace(const StepParams &p, int s, in
                 c[k] = __ldcs(cin + i);
                 q[k] = __ldcs(vin + i);
             }
+        }
+        // the warp's next tile on its way to L2 (20 lines of 128 bytes, a lane each): the
+        // few warps that the histograms leave resident do not cover HBM's latency
+        if (lane < 20 && t + kNW < w1) {
+            const long long nb = base + (long long)kNW * kWT;
+            const long long i = lane < 16 ? nb + 8 * lane : nb + 32 * (lane - 16);
+            if (i < n)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(lane < 16 ? (const void *)(vin + i)
+                                                                        : (const void *)(cin + i)));
         }
 #pragma unroll
         for (int k = 0; k < kWI; ++k) {
@@ -474,14 +484,74 @@ size_t particle_tma_smem_bytes(int nn, int stages)
     return (size_t)16 * stages + (size_t)stages * kTmaTile * 20 + (size_t)nn * 4 * sizeof(unsigned);
 }
 
-// slots [r0, r1) of a species of n particles for CTA `cta` of `nctas`: equal shares to
+// slots [r0, r1) of a species of n particles from f0 to f1 of `parts`: equal shares to
 // within 4 slots (a multiple of 4 at every boundary, so that each tile's cells start on
 // a 16-byte boundary), walked in tiles of kTmaTile from r0 (the last one partial).  A
 // share of whole tiles would leave some CTAs a tile more than others.
-__device__ __forceinline__ void tma_share(long long n, int cta, int nctas, long long &r0, long long &r1)
+__device__ __forceinline__ void tma_share(long long n, int f0, int f1, int parts, long long &r0, long long &r1)
 {
-    r0 = (n * cta / nctas) & ~3LL;
-    r1 = cta + 1 == nctas ? n : (n * (cta + 1) / nctas) & ~3LL;
+    r0 = (n * f0 / parts) & ~3LL;
+    r1 = f1 == parts ? n : (n * f1 / parts) & ~3LL;
+}
+
+// The producer's lane for slots [r0, r1) of a species: its tiles into the ring, the k-th tile
+// of the CTA into stage k mod stages.  Returns false once a wait has given up.
+__device__ __forceinline__ bool tma_produce(const int32_t *cin, const float4 *vin, long long r0, long long r1,
+                                            long long &k, int stages, uint64_t *full, uint64_t *empty,
+                                            float4 *s_v, int32_t *s_c, volatile int *fail, int *error,
+                                            long long wait_cycles)
+{
+    for (long long i0 = r0; i0 < r1; i0 += kTmaTile, ++k) {
+        const int st = (int)(k % stages);
+        const unsigned ph = (unsigned)((k / stages) & 1);
+        if (k >= stages && !mbar_wait(&empty[st], ph ^ 1u, fail, error, wait_cycles))
+            return false;
+        const int cnt = (int)min((long long)kTmaTile, r1 - i0);
+        const int cb = cnt & ~3;  // cells by bulk copy (16-byte multiple)
+        mbar_expect_tx(&full[st], (unsigned)(cnt * 16 + cb * 4));
+        bulk_load(s_v + (size_t)st * kTmaTile, vin + i0, (unsigned)cnt * 16, &full[st]);
+        if (cb)
+            bulk_load(s_c + (size_t)st * kTmaTile, cin + i0, (unsigned)cb * 4, &full[st]);
+    }
+    return true;
+}
+
+// every copy issued has landed before the CTA may exit (also after a wait of the
+// pipeline gave up)
+__device__ __forceinline__ void tma_drain(long long k, int stages, uint64_t *full, int *error)
+{
+    for (long long j = (k > stages ? k - stages : 0); j < k; ++j)
+        if (!mbar_drain(&full[j % stages], (unsigned)((j / stages) & 1), error))
+            break;
+}
+
+// A species' share done (consumers only): absorbed counts, histogram flush and clear
+__device__ __forceinline__ void tma_flush(const StepParams &p, int s, int P, unsigned nabs0, unsigned nabs1,
+                                          unsigned *s_lo, unsigned *s_hi, unsigned *s_abs)
+{
+    const unsigned a0 = __reduce_add_sync(0xffffffffu, nabs0);
+    const unsigned a1 = __reduce_add_sync(0xffffffffu, nabs1);
+    if ((threadIdx.x & 31) == 0) {
+        if (a0)
+            atomicAdd(&s_abs[0], a0);
+        if (a1)
+            atomicAdd(&s_abs[1], a1);
+    }
+    consumers_sync();
+    unsigned long long *acc = p.acc + ((size_t)(P ^ 1) * p.ns + s) * p.nn;
+    for (int j = threadIdx.x; j < p.nn; j += kTmaConsumers) {
+        const unsigned long long v = ((unsigned long long)s_hi[j] << 32) + s_lo[j];
+        if (v)
+            atomicAdd(acc + j, v);
+        s_lo[j] = 0u;
+        s_hi[j] = 0u;
+    }
+    if (threadIdx.x < 2) {
+        if (s_abs[threadIdx.x])
+            atomicAdd(&p.st->absorbed_step[s][threadIdx.x], (unsigned long long)s_abs[threadIdx.x]);
+        s_abs[threadIdx.x] = 0u;
+    }
+    consumers_sync();
 }
 
 // One species' share of the in-place TMA step, for a consumer thread: its tiles from
@@ -495,16 +565,14 @@ __device__ __forceinline__ void tma_species(const StepParams &p, int s, int P, i
                                             const float4 *s_v, const int32_t *s_c,
                                             const float *s_E, const float *s_lam,
                                             DepositSplit32 &dep, volatile int *fail,
-                                            unsigned &nabs0, unsigned &nabs1)
+                                            unsigned &nabs0, unsigned &nabs1, long long r0,
+                                            long long r1)
 {
     const SpeciesDev &sp = p.sp[s];
     const int lane = threadIdx.x & 31;
-    const long long n = (long long)*(volatile unsigned long long *)&p.st->count[s][P];
     const int32_t *__restrict__ cin = sp.cell[P];
     int32_t *__restrict__ cout = sp.cell[P ^ 1];
     float4 *__restrict__ vout = sp.pv[P ^ 1];
-    long long r0, r1;
-    tma_share(n, blockIdx.x, gridDim.x, r0, r1);
     for (long long i0 = r0; i0 < r1; i0 += kTmaTile) {
         const bool ok = !*fail && mbar_wait(&full[st], ph, fail, &p.st->error, p.wait_cycles);
         const int cnt = (int)min((long long)kTmaTile, r1 - i0);
@@ -617,27 +685,12 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_particles_tma(const __grid_c
                 const SpeciesDev &sp = p.sp[s];
                 const long long n = (long long)*(volatile unsigned long long *)&p.st->count[s][P];
                 long long r0, r1;
-                tma_share(n, blockIdx.x, gridDim.x, r0, r1);
-                for (long long i0 = r0; i0 < r1; i0 += kTmaTile, ++k) {
-                    const int st = (int)(k % stages);
-                    const unsigned ph = (unsigned)((k / stages) & 1);
-                    if (k >= stages &&
-                        !mbar_wait(&empty[st], ph ^ 1u, fail, &p.st->error, p.wait_cycles))
-                        break;
-                    const int cnt = (int)min((long long)kTmaTile, r1 - i0);
-                    const int cb = cnt & ~3;  // cells by bulk copy (16-byte multiple)
-                    mbar_expect_tx(&full[st], (unsigned)(cnt * 16 + cb * 4));
-                    bulk_load(s_v + (size_t)st * kTmaTile, sp.pv[P] + i0, (unsigned)cnt * 16, &full[st]);
-                    if (cb)
-                        bulk_load(s_c + (size_t)st * kTmaTile, sp.cell[P] + i0, (unsigned)cb * 4,
-                                  &full[st]);
-                }
-            }
-            // every copy issued has landed before the CTA may exit (also after a wait
-            // of the pipeline gave up)
-            for (long long j = (k > stages ? k - stages : 0); j < k; ++j)
-                if (!mbar_drain(&full[j % stages], (unsigned)((j / stages) & 1), &p.st->error))
+                tma_share(n, blockIdx.x, blockIdx.x + 1, gridDim.x, r0, r1);
+                if (!tma_produce(sp.cell[P], sp.pv[P], r0, r1, k, stages, full, empty, s_v, s_c, fail,
+                                 &p.st->error, p.wait_cycles))
                     break;
+            }
+            tma_drain(k, stages, full, &p.st->error);
         }
     } else {
         // ---- consumers
@@ -647,41 +700,20 @@ __global__ void __launch_bounds__(kTmaThreads, 1) k_particles_tma(const __grid_c
             const SpeciesDev &sp = p.sp[s];
             DepositSplit32 dep{s_lo, s_hi};
             unsigned nabs0 = 0u, nabs1 = 0u;
+            const long long n = (long long)*(volatile unsigned long long *)&p.st->count[s][P];
+            long long r0, r1;
+            tma_share(n, blockIdx.x, blockIdx.x + 1, gridDim.x, r0, r1);
             // the species' tiles: the sheath's common shape (Heaviside beta between
             // plates) with both fixed at compile time, every other shape read at run
             // time (the same arithmetic either way)
             if (sp.kind == SLPIC_BETA_HEAVISIDE && !p.periodic)
                 tma_species<kProf, SLPIC_BETA_HEAVISIDE, 0>(p, s, P, st, ph, stages, full, empty,
                                                            s_v, s_c, s_E, s_lam, dep, fail, nabs0,
-                                                           nabs1);
+                                                           nabs1, r0, r1);
             else
                 tma_species<kProf, kAny, kAny>(p, s, P, st, ph, stages, full, empty, s_v, s_c,
-                                               s_E, s_lam, dep, fail, nabs0, nabs1);
-            // species done: absorbed counts, histogram flush and clear
-            const unsigned a0 = __reduce_add_sync(0xffffffffu, nabs0);
-            const unsigned a1 = __reduce_add_sync(0xffffffffu, nabs1);
-            if (lane == 0) {
-                if (a0)
-                    atomicAdd(&s_abs[0], a0);
-                if (a1)
-                    atomicAdd(&s_abs[1], a1);
-            }
-            consumers_sync();
-            unsigned long long *acc = p.acc + ((size_t)(P ^ 1) * p.ns + s) * p.nn;
-            for (int j = threadIdx.x; j < p.nn; j += kTmaConsumers) {
-                const unsigned long long v = ((unsigned long long)s_hi[j] << 32) + s_lo[j];
-                if (v)
-                    atomicAdd(acc + j, v);
-                s_lo[j] = 0u;
-                s_hi[j] = 0u;
-            }
-            if (threadIdx.x < 2) {
-                if (s_abs[threadIdx.x])
-                    atomicAdd(&p.st->absorbed_step[s][threadIdx.x],
-                              (unsigned long long)s_abs[threadIdx.x]);
-                s_abs[threadIdx.x] = 0u;
-            }
-            consumers_sync();
+                                               s_E, s_lam, dep, fail, nabs0, nabs1, r0, r1);
+            tma_flush(p, s, P, nabs0, nabs1, s_lo, s_hi, s_abs);
         }
     }
     span_exit(p.st, 0);
@@ -707,9 +739,9 @@ __global__ void __launch_bounds__(kPB, 3) k_particles_compact(const __grid_const
 {
     span_enter(p.st, 0);
     if (p.sp[blockIdx.y].kind == SLPIC_BETA_HEAVISIDE && !p.periodic)
-        particles_compact<kProf, SLPIC_BETA_HEAVISIDE, 0>(p, blockIdx.y, blockIdx.x, gridDim.x);
+        particles_compact<kProf, SLPIC_BETA_HEAVISIDE, 0>(p, blockIdx.y, blockIdx.x, blockIdx.x + 1, gridDim.x);
     else
-        particles_compact<kProf>(p, blockIdx.y, blockIdx.x, gridDim.x);
+        particles_compact<kProf>(p, blockIdx.y, blockIdx.x, blockIdx.x + 1, gridDim.x);
     span_exit(p.st, 0);
 }
 
@@ -718,29 +750,137 @@ __global__ void __launch_bounds__(kPB, 4) k_particles(const __grid_constant__ St
 {
     span_enter(p.st, 0);
     if (p.sp[blockIdx.y].kind == SLPIC_BETA_HEAVISIDE && !p.periodic)
-        particles_inplace<kProf, SLPIC_BETA_HEAVISIDE, 0>(p, blockIdx.y, blockIdx.x, gridDim.x);
+        particles_inplace<kProf, SLPIC_BETA_HEAVISIDE, 0>(p, blockIdx.y, blockIdx.x, blockIdx.x + 1, gridDim.x);
     else
-        particles_inplace<kProf>(p, blockIdx.y, blockIdx.x, gridDim.x);
+        particles_inplace<kProf>(p, blockIdx.y, blockIdx.x, blockIdx.x + 1, gridDim.x);
     span_exit(p.st, 0);
 }
 
 // Batched forms: CTA b works on (instance, species, share, shares) = work[b].
-__global__ void __launch_bounds__(kPB, 3)
-    k_particles_compact_batch(const StepParams *__restrict__ ps, const int4 *__restrict__ work)
+// Batched: CTA b walks work items first[b] .. first[b+1]-1, each {instance, species, f0, f1}: the
+// instance's tiles of that species from f0 to f1 of kBatchParts.  The items are cut so that
+// every CTA has the same number of particles, whatever the instances' sizes; one CTA per item of
+// about equal sizes left 962 CTAs on 608 places, the second wave half empty (885 us a step of 48
+// sheaths, 68 million particles; 840 with this and the L2 prefetch).  In place this form takes
+// the grids with no room for the ring of k_particles_batch_tma.
+template <bool kCompact>
+__device__ __forceinline__ void batch_items(const StepParams *__restrict__ ps, const int4 *__restrict__ work,
+                                            const int *__restrict__ first)
 {
     __shared__ StepParams s_p;
-    const int4 w = work[blockIdx.x];
-    load_params(s_p, ps + w.x);
-    particles_compact<false>(s_p, w.y, w.z, w.w);
+    for (int i = first[blockIdx.x], end = first[blockIdx.x + 1]; i < end; ++i) {
+        const int4 w = work[i];
+        __syncthreads();  // the item before has left the shared memory
+        load_params(s_p, ps + w.x);
+        if (kCompact)
+            particles_compact<false>(s_p, w.y, w.z, w.w, kBatchParts);
+        else
+            particles_inplace<false>(s_p, w.y, w.z, w.w, kBatchParts);
+    }
+}
+
+__global__ void __launch_bounds__(kPB, 3)
+    k_particles_compact_batch(const StepParams *__restrict__ ps, const int4 *__restrict__ work,
+                              const int *__restrict__ first)
+{
+    batch_items<true>(ps, work, first);
 }
 
 __global__ void __launch_bounds__(kPB, 4)
-    k_particles_batch(const StepParams *__restrict__ ps, const int4 *__restrict__ work)
+    k_particles_batch(const StepParams *__restrict__ ps, const int4 *__restrict__ work,
+                      const int *__restrict__ first)
 {
+    batch_items<false>(ps, work, first);
+}
+
+// The batched in-place step with the TMA-staged stream (see k_particles_tma), one CTA per SM:
+// the ring runs on across the CTA's items (the producer reads the next item's
+// parameters from global memory while the consumers finish the one before), the
+// consumers exchange parameters, field and histogram between items.  Issue-bound like
+// k_particles_tma; 620 us a step of 48 sheaths (68 million particles) against 840 of the
+// per-warp form, whose warps waited for their loads (issue slots 64% used).
+__global__ void __launch_bounds__(kTmaThreads, 1)
+    k_particles_batch_tma(const StepParams *__restrict__ ps, const int4 *__restrict__ work,
+                          const int *__restrict__ first, int max_nn, int stages)
+{
+    extern __shared__ __align__(16) unsigned char smem[];
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem);
+    uint64_t *empty = full + stages;
+    float4 *s_v = reinterpret_cast<float4 *>(smem + 16 * stages);
+    int32_t *s_c = reinterpret_cast<int32_t *>(s_v + (size_t)stages * kTmaTile);
+    unsigned *s_lo = reinterpret_cast<unsigned *>(s_c + (size_t)stages * kTmaTile);
+    unsigned *s_hi = s_lo + max_nn;
+    float *s_E = reinterpret_cast<float *>(s_hi + max_nn);
     __shared__ StepParams s_p;
-    const int4 w = work[blockIdx.x];
-    load_params(s_p, ps + w.x);
-    particles_inplace<false>(s_p, w.y, w.z, w.w);
+    __shared__ unsigned s_abs[2];
+    __shared__ int s_fail;
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    for (int j = threadIdx.x; j < max_nn; j += kTmaThreads) {
+        s_lo[j] = 0u;
+        s_hi[j] = 0u;
+    }
+    if (threadIdx.x == 0) {
+        for (int k = 0; k < stages; ++k) {
+            mbar_init(&full[k], 1);
+            mbar_init(&empty[k], kTmaConsumers / 32);
+        }
+        s_abs[0] = s_abs[1] = 0u;
+        s_fail = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    __syncthreads();
+    volatile int *fail = &s_fail;
+    const int i0 = first[blockIdx.x], i1 = first[blockIdx.x + 1];
+    if (warp == kTmaConsumers / 32) {
+        if (lane == 0 && i0 < i1) {
+            long long k = 0;
+            for (int i = i0; i < i1 && !*fail; ++i) {
+                const int4 w = work[i];
+                const StepParams *p = ps + w.x;
+                const int P = (int)(*(volatile long long *)&p->st->step & 1);
+                const long long n = (long long)*(volatile unsigned long long *)&p->st->count[w.y][P];
+                long long r0, r1;
+                tma_share(n, w.z, w.w, kBatchParts, r0, r1);
+                if (!tma_produce(p->sp[w.y].cell[P], p->sp[w.y].pv[P], r0, r1, k, stages, full, empty, s_v,
+                                 s_c, fail, &p->st->error, p->wait_cycles))
+                    break;
+            }
+            tma_drain(k, stages, full, &ps[work[i1 - 1].x].st->error);
+        }
+        return;
+    }
+    int st = 0;        // stage of the next tile
+    unsigned ph = 0u;  // its phase
+    static_assert(sizeof(StepParams) % 8 == 0, "copied as 8-byte words");
+    for (int i = i0; i < i1; ++i) {
+        const int4 w = work[i];
+        {
+            const unsigned long long *a = reinterpret_cast<const unsigned long long *>(ps + w.x);
+            unsigned long long *b = reinterpret_cast<unsigned long long *>(&s_p);
+            for (int k = threadIdx.x; k < (int)(sizeof(StepParams) / 8); k += kTmaConsumers)
+                b[k] = a[k];
+        }
+        consumers_sync();
+        const StepParams &p = s_p;
+        const int s = w.y;
+        const int P = (int)(*(volatile long long *)&p.st->step & 1);
+        const long long n = (long long)*(volatile unsigned long long *)&p.st->count[s][P];
+        for (int j = threadIdx.x; j < p.nn; j += kTmaConsumers)
+            s_E[j] = p.E[j];
+        consumers_sync();
+        long long r0, r1;
+        tma_share(n, w.z, w.w, kBatchParts, r0, r1);
+        DepositSplit32 dep{s_lo, s_hi};
+        unsigned nabs0 = 0u, nabs1 = 0u;
+        if (p.sp[s].kind == SLPIC_BETA_HEAVISIDE && !p.periodic)
+            tma_species<false, SLPIC_BETA_HEAVISIDE, 0>(p, s, P, st, ph, stages, full, empty, s_v, s_c, s_E,
+                                                       s_E, dep, fail, nabs0, nabs1, r0, r1);
+        else
+            tma_species<false, kAny, kAny>(p, s, P, st, ph, stages, full, empty, s_v, s_c, s_E, s_E, dep,
+                                           fail, nabs0, nabs1, r0, r1);
+        tma_flush(p, s, P, nabs0, nabs1, s_lo, s_hi, s_abs);
+    }
 }
 
 // ---------------------------------------------------------------------------------
@@ -851,13 +991,63 @@ __global__ void __launch_bounds__(256) k_hard(const __grid_constant__ StepParams
     span_exit(p.st, 1);
 }
 
-// batched: grid (CTAs per instance, instances)
-__global__ void __launch_bounds__(256) k_hard_batch(const StepParams *__restrict__ ps, int compact)
+// batched: the instances' lists as one index space of chunks of 256 (an instance's last one
+// partial), dealt out to the CTAs in turn, whatever the instances' shares of the walks.  A
+// fixed number of CTAs per instance waited for the instance with the longest list: 125 us a
+// step of 48 sheaths, now 59.
+__global__ void __launch_bounds__(256) k_hard_batch(const StepParams *__restrict__ ps, int m, int compact)
 {
     __shared__ StepParams s_p;
-    load_params(s_p, ps + blockIdx.y);
-    hard_body<false>(s_p, compact, (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5),
-              (long long)gridDim.x * (blockDim.x >> 5));
+    __shared__ int s_pre[257], s_warp[8];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    int have = -1;
+    long long base = 0;  // chunks of the instances before this group of 256
+    for (int g = 0; g < m; g += 256) {
+        int n = 0;
+        if (g + (int)threadIdx.x < m) {
+            const StepParams *p = ps + g + threadIdx.x;
+            unsigned long long k = 0;
+            for (int s = 0; s < p->ns; ++s)
+                k += *(volatile unsigned long long *)&p->st->hard_n[s];
+            n = (int)((k + 255) / 256);
+        }
+        int incl = n;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int v = __shfl_up_sync(0xffffffffu, incl, d);
+            if (lane >= d)
+                incl += v;
+        }
+        __syncthreads();  // the group before has left s_pre and s_warp
+        if (lane == 31)
+            s_warp[warp] = incl;
+        __syncthreads();
+        for (int w = 0; w < warp; ++w)
+            incl += s_warp[w];
+        s_pre[threadIdx.x + 1] = incl;
+        if (threadIdx.x == 0)
+            s_pre[0] = 0;
+        __syncthreads();
+        const int total = s_pre[256];
+        const long long r = (base + gridDim.x - 1 - blockIdx.x) / gridDim.x;  // turns before the group
+        for (long long c = r * gridDim.x + blockIdx.x - base; c < total; c += gridDim.x) {
+            int lo = 0, hi = 256;  // s_pre[lo] <= c < s_pre[hi]
+            while (hi - lo > 1) {
+                const int mid = (lo + hi) >> 1;
+                if (s_pre[mid] <= c)
+                    lo = mid;
+                else
+                    hi = mid;
+            }
+            if (g + lo != have) {
+                have = g + lo;
+                __syncthreads();  // the chunk before has left the parameters
+                load_params(s_p, ps + have);
+            }
+            hard_body<false>(s_p, compact, (c - s_pre[lo]) * 8 + warp, 1LL << 40);
+        }
+        base += total;
+    }
 }
 
 // ---------------------------------------------------------------------------------
@@ -1689,20 +1879,29 @@ void launch_hard(const StepParams &p, int ctas, bool compact, cudaStream_t st)
     (p.lam ? k_hard<true> : k_hard<false>)<<<ctas, 256, 0, st>>>(p, compact ? 1 : 0);
 }
 
-void launch_particles_batch(const StepParams *d_params, const int4 *d_work, int n_work,
-                            int max_nn, bool compact, cudaStream_t st)
+// the ring's bytes, the histogram's two words and E per node
+static size_t batch_tma_smem_bytes(int nn, int stages)
 {
-    if (compact)
-        k_particles_compact_batch<<<n_work, kPB, particle_kernel_smem_bytes(max_nn), st>>>(d_params,
-                                                                                          d_work);
-    else
-        k_particles_batch<<<n_work, kPB, particle_inplace_smem_bytes(max_nn), st>>>(d_params, d_work);
+    return (size_t)16 * stages + (size_t)stages * kTmaTile * 20 + (size_t)nn * 3 * sizeof(unsigned);
 }
 
-void launch_hard_batch(const StepParams *d_params, int m, int ctas_per_instance, bool compact,
-                       cudaStream_t st)
+void launch_particles_batch(const StepParams *d_params, const BatchWork &w, int max_nn, bool compact,
+                            int stages, cudaStream_t st)
 {
-    k_hard_batch<<<dim3(ctas_per_instance, m), 256, 0, st>>>(d_params, compact ? 1 : 0);
+    if (compact)
+        k_particles_compact_batch<<<w.ctas, kPB, particle_kernel_smem_bytes(max_nn), st>>>(
+            d_params, w.items, w.first);
+    else if (stages)
+        k_particles_batch_tma<<<w.ctas, kTmaThreads, batch_tma_smem_bytes(max_nn, stages), st>>>(
+            d_params, w.items, w.first, max_nn, stages);
+    else
+        k_particles_batch<<<w.ctas, kPB, particle_inplace_smem_bytes(max_nn), st>>>(d_params, w.items,
+                                                                                    w.first);
+}
+
+void launch_hard_batch(const StepParams *d_params, int m, int ctas, bool compact, cudaStream_t st)
+{
+    k_hard_batch<<<ctas, 256, 0, st>>>(d_params, m, compact ? 1 : 0);
 }
 
 void launch_field_batch(const StepParams *d_params, int m, int max_nn, int max_ns, int mode,
@@ -1711,9 +1910,30 @@ void launch_field_batch(const StepParams *d_params, int m, int max_nn, int max_n
     k_field_batch<<<m * kFC, kFCT, field_cluster_smem_bytes(max_nn, max_ns, kFC), st>>>(d_params, mode);
 }
 
-cudaError_t configure_batch_kernels(int max_nn, int *inplace_per_sm, int *compact_per_sm)
+cudaError_t configure_batch_kernels(int max_nn, int *inplace_per_sm, int *compact_per_sm, int *stages)
 {
-    cudaError_t e = cudaFuncSetAttribute(k_particles_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    *stages = 0;
+    int dev = 0, optin = 0;
+    cudaFuncAttributes at;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess)
+        e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess)
+        e = cudaFuncGetAttributes(&at, k_particles_batch_tma);
+    if (e != cudaSuccess)
+        return e;
+    // the TMA-staged kernel where two stages of its ring or more fit beside the grid
+    int k = 4;
+    while (k >= 2 && batch_tma_smem_bytes(max_nn, k) + at.sharedSizeBytes > (size_t)optin)
+        --k;
+    if (k >= 2) {
+        *stages = k;
+        e = cudaFuncSetAttribute(k_particles_batch_tma, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)batch_tma_smem_bytes(max_nn, k));
+        if (e != cudaSuccess)
+            return e;
+    }
+    e = cudaFuncSetAttribute(k_particles_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)particle_inplace_smem_bytes(max_nn));
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(k_particles_compact_batch,
@@ -1728,6 +1948,10 @@ cudaError_t configure_batch_kernels(int max_nn, int *inplace_per_sm, int *compac
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(compact_per_sm, k_particles_compact_batch,
                                                           kPB, particle_kernel_smem_bytes(max_nn));
+    // (its CTA counts as two: with a part per resident CTA and wave the parts of the default two
+    // waves balance worse than those of four, 762 against 732 us a step of 48 sheaths)
+    if (*stages)
+        *inplace_per_sm = 2;
     return e;
 }
 

@@ -58,13 +58,21 @@ void launch_snapshot(const unsigned long long *dep, unsigned long long *dep_out,
 // rho and phi (p.rho, p.phi) from the deposit dep ([species][nn]) of time level step
 void launch_potential(const StepParams &p, const unsigned long long *dep, long long step,
                       cudaStream_t st);
-// batched forms over many instances: d_params[m] on the device; the particle
-// kernels take one CTA per work item (instance, species, share, shares)
-cudaError_t configure_batch_kernels(int max_nn, int *inplace_per_sm, int *compact_per_sm);
-void launch_particles_batch(const StepParams *d_params, const int4 *d_work, int n_work,
-                            int max_nn, bool compact, cudaStream_t st);
-void launch_hard_batch(const StepParams *d_params, int m, int ctas_per_instance, bool compact,
-                       cudaStream_t st);
+// batched forms over many instances: d_params[m] on the device.  A CTA b of a particle
+// kernel takes the work items first[b] .. first[b+1]-1, {instance, species, f0, f1} each: the
+// instance's tiles of that species from f0 to f1 of kBatchParts.
+constexpr int kBatchParts = 1 << 24;
+struct BatchWork {
+    int4 *items = nullptr;
+    int *first = nullptr;
+    int ctas = 0;
+};
+// CTAs per SM of the batched particle kernels; stages: of the TMA-staged in-place one (0: the
+// per-warp one)
+cudaError_t configure_batch_kernels(int max_nn, int *inplace_per_sm, int *compact_per_sm, int *stages);
+void launch_particles_batch(const StepParams *d_params, const BatchWork &w, int max_nn, bool compact,
+                            int stages, cudaStream_t st);
+void launch_hard_batch(const StepParams *d_params, int m, int ctas, bool compact, cudaStream_t st);
 void launch_field_batch(const StepParams *d_params, int m, int max_nn, int max_ns, int mode,
                         cudaStream_t st);
 void launch_deposit(const StepParams &p, int ctas_per_species, cudaStream_t st);
