@@ -826,7 +826,9 @@ def run_2d(args):
                         "cg_rel_residual_last": d1["cg_rel_residual"],
                         "cold_start_iterations": d_prep["cg_iterations"],
                         "ms_per_step": fk, "load_and_first_solve_s": prep_s},
-        "cpu_baseline": cpu, "gpu_launches": 3 * args.steps, "clocks": clocks.summary(),
+        "cpu_baseline": cpu,
+        # particles 2, source 2, and the solve: 4 (direct) or 1 (CG); the sorts not counted
+        "gpu_launches": (8 if args.solver == "fft" else 5) * args.steps, "clocks": clocks.summary(),
     }
     print(json.dumps(line), flush=True)
     sim.close()
@@ -1127,7 +1129,11 @@ def run_paper_sheath(args):
             acc = [acc[0] + phi, acc[1] + sim.density(0), acc[2] + sim.density(1)]
             m += 1
         sim.close()
-        res[name] = {"steps": n, "dt": prob["dt"], "ms": ms, "us_per_step": 1e3 * ms / n,
+        # a simulation of up to 7 million slots takes up to 4,096 steps a launch, a larger
+        # one three launches a step
+        slots = sum(sp["capacity"] for sp in prob["species"])
+        res[name] = {"steps": n, "launches": -(-n // 4096) if slots <= 7_000_000 else 3 * n,
+                     "dt": prob["dt"], "ms": ms, "us_per_step": 1e3 * ms / n,
                      "macroparticles_end": d["count"][:2],
                      "profiles": [a / m for a in acc]}
     pic, sl = res["pic"], res["slpic"]
@@ -1155,7 +1161,7 @@ def run_paper_sheath(args):
                   "macroparticles_end": sl["macroparticles_end"]},
         "steady_state_agreement": {"max_dphi_over_bias": dphi_max,
                                    "max_dn_e_over_peak": dens[0], "max_dn_i_over_peak": dens[1]},
-        "gpu_launches": 3 * (pic["steps"] + sl["steps"]),
+        "gpu_launches": pic["launches"] + sl["launches"],
         "note": "the paper's 160x is VSim on unstated CPU hardware: context, not the target",
     }
     print(json.dumps(line), flush=True)

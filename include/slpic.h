@@ -202,7 +202,7 @@ int slpic_prepare(slpic_t *h);
  * rho^{n+1}; then inject source particles (deposited into rho^{n+1}, first
  * pushed next step) and solve phi^{n+1}, E^{n+1}.  The steps run as a
  * captured CUDA graph with no host synchronisation between them; a call of 4 or
- * more steps of a simulation of at most 15 million slots (capacities) runs them
+ * more steps of a simulation of at most 7 million slots (capacities) runs them
  * in one launch instead (at most 4096 steps each), with the same results. */
 int slpic_step(slpic_t *h, int64_t nsteps);
 

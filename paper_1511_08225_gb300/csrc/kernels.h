@@ -41,9 +41,9 @@ void launch_particles_tma(const StepParams &p, int ctas, int stages, cudaStream_
 // steps_scratch_bytes on the device; max_smem: dynamic shared memory it may take
 constexpr int kStepsThreads = 1024;
 // Where the line lies (us a step, three kernels against k_steps): 2,560 particles 27 / 9,
-// 51,200 30 / 12, 5.2e5 42 / 25, 2.0e6 62 / 47, 4.9e6 83 / 75 (14.7M slots), 8.2e6 112 /
-// 114.  The host knows the slots, of which a third to all are in use.
-constexpr long long kStepsMaxSlots = 15000000;        // most slots, all species
+// 51,200 30 / 12, 5.2e5 42 / 25, 2.0e6 62 / 47, 4.9e6 83 / 75, 8.1e6 104 / 107.5.  The host
+// knows the slots, of which a third to all are in use: at 7e6 it is no slower for any count.
+constexpr long long kStepsMaxSlots = 7000000;         // most slots, all species
 constexpr long long kStepsMaxSpecies = (1LL << 24) - 1;  // ... and of one: its sums fit 64 bits
 constexpr int kStepsFewest = 4, kStepsMost = 4096;  // steps of a launch
 size_t steps_scratch_bytes(int nn, int ns);
