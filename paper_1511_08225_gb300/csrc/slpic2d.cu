@@ -1605,9 +1605,10 @@ constexpr int kFinishThreads = 128;
 // 1 where that leaves fewer than 512 warps (3 an SM), too few to hide the FP64 latency.  The
 // solve of a step with 1 and with 3: 64 x 64 37.2 and 45.4 us, 64 x 1,000 (250 warps with 3)
 // 59.6 and 65.3, 256^2 52.4 and 57.8, 512^2 (1,022) 104.5 and 93.9, 1,024^2 316 and 299.
+// Rows of fewer than 8 points always 1: they do not fill a thread's 8.
 int fft_levels(int nx, int ny)
 {
-    return ((long long)(ny - 1) * nx >> 8) < 512 ? 1 : 3;
+    return nx < 8 || ((long long)(ny - 1) * nx >> 8) < 512 ? 1 : 3;
 }
 // threads of a row's transform, and rows of a CTA (a warp at least)
 __host__ __device__ __forceinline__ int fft_row_threads(int nx, int levels)
@@ -1831,7 +1832,7 @@ __global__ void __launch_bounds__(kFftMaxThreads) k_fft_rows(const __grid_consta
     __syncthreads();
     const double *bq = p.q + row;
     double2 *out = p.spec + row;
-    const bool one = T * N >= nx;  // the row is in registers
+    const bool one = T * N == nx;  // the row is in registers, a thread's point q T after its first in b[q]
     fft_row<LV, R0, false>(
         x, p.tw, nx, t, T, p.log2nx,
         [&](int i, int q) { return make_double2(one ? b[q] : act ? bq[i] : 0.0, 0.0); },
