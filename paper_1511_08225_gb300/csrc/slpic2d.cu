@@ -32,6 +32,7 @@
 
 #include "push_math.cuh"
 #include "slpic2d.h"
+#include "smem_limit.h"
 #include "unet_internal.h"
 
 namespace slpic {
@@ -2728,19 +2729,14 @@ extern "C" int slpic2d_create(const slpic2d_config *c, slpic2d_t **out)
         if (e2 == cudaSuccess)
             e2 = cudaMemset(p.finished, 0, sizeof(unsigned));
         const size_t tri = tri_smem_bytes(p.ny);
-        int most = 0;
-        cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-        if (e2 == cudaSuccess && tri + sizeof(TriEnds) <= (size_t)most) {
+        if (e2 == cudaSuccess && allow_dynamic_smem(k_tridiag_modes<true>, tri) == cudaSuccess)
             h->tri_smem = tri;
-            if (tri > 32 * 1024)
-                e2 = cudaFuncSetAttribute(k_tridiag_modes<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          (int)tri);
-        }
-        const int smem = 16 * p.nx * fft_cta_rows(p.nx, fft_levels(p.nx, p.ny));
-        if (e2 == cudaSuccess && smem > 48 * 1024)
-            e2 = cudaFuncSetAttribute(fft_kernel(p), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-        if (e2 == cudaSuccess && smem > 48 * 1024)
-            e2 = cudaFuncSetAttribute(ifft_kernel(p), cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        cudaGetLastError();
+        const size_t smem = (size_t)16 * p.nx * fft_cta_rows(p.nx, fft_levels(p.nx, p.ny));
+        if (e2 == cudaSuccess)
+            e2 = allow_dynamic_smem(fft_kernel(p), smem);
+        if (e2 == cudaSuccess)
+            e2 = allow_dynamic_smem(ifft_kernel(p), smem);
         if (e2 != cudaSuccess)
             return bail(SLPIC_ERR_CUDA, cudaGetErrorString(e2));
     }
