@@ -18,6 +18,7 @@
 #include "particle_step.cuh"
 #include "push_math.cuh"
 #include "slpic_internal.cuh"
+#include "smem_limit.h"
 
 namespace slpic {
 
@@ -1928,20 +1929,15 @@ cudaError_t configure_batch_kernels(int max_nn, int *inplace_per_sm, int *compac
         --k;
     if (k >= 2) {
         *stages = k;
-        e = cudaFuncSetAttribute(k_particles_batch_tma, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)batch_tma_smem_bytes(max_nn, k));
+        e = allow_dynamic_smem(k_particles_batch_tma, batch_tma_smem_bytes(max_nn, k));
         if (e != cudaSuccess)
             return e;
     }
-    e = cudaFuncSetAttribute(k_particles_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)particle_inplace_smem_bytes(max_nn));
+    e = allow_dynamic_smem(k_particles_batch, particle_inplace_smem_bytes(max_nn));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_particles_compact_batch,
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)particle_kernel_smem_bytes(max_nn));
+        e = allow_dynamic_smem(k_particles_compact_batch, particle_kernel_smem_bytes(max_nn));
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_field_batch, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)field_cluster_smem_bytes(max_nn, kMaxSpecies, kFC));
+        e = allow_dynamic_smem(k_field_batch, field_cluster_smem_bytes(max_nn, kMaxSpecies, kFC));
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(inplace_per_sm, k_particles_batch, kPB,
                                                           particle_inplace_smem_bytes(max_nn));

@@ -5,7 +5,7 @@ gives alone."""
 import numpy as np
 import pytest
 
-from paper_1511_08225_gb300 import binding2d, inputs
+from paper_1511_08225_gb300 import binding, binding2d, inputs
 
 pytestmark = pytest.mark.gpu
 
@@ -37,3 +37,25 @@ def test_direct_solver_with_a_smaller_grid_beside_it(large, small):
         for a, b in zip(mine, _direct_run(alone, r)):
             assert np.array_equal(a, b)
         alone.close()
+
+
+def _batch_run(b, probs, states):
+    for i, st in enumerate(states):
+        b.load_state(i, st)
+    b.prepare()
+    b.step(18)  # past a compacting step
+    out = [f for i in range(len(probs)) for f in b.fields(i)]
+    b.close()
+    return out
+
+
+# in place: the staged kernel beside 11,000 nodes, the per-warp kernel at 15,000
+@pytest.mark.parametrize("cells", [11000, 15000])
+def test_batch_with_a_smaller_batch_beside_it(cells):
+    probs = [[inputs.sheath_problem(n_cells=n, ppc=20, v0=0.05) for n in sizes] for sizes in ((cells, 70), (60, 50))]
+    states = [[inputs.load_state(p) for p in ps] for ps in probs]
+    batches = [binding.Batch(ps) for ps in probs]
+    got = [_batch_run(*a) for a in zip(batches, probs, states)]
+    for ps, st, mine in zip(probs, states, got):
+        for a, b in zip(mine, _batch_run(binding.Batch(ps), ps, st)):
+            assert np.array_equal(a, b)
