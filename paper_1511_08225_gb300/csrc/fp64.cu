@@ -30,6 +30,7 @@
 #include <cuda_runtime.h>
 
 #include "slpic_fp64.h"
+#include "smem_limit.h"
 
 namespace slpic {
 int check_config(const slpic_config *c, std::string &why);  // api.cu
@@ -767,7 +768,7 @@ extern "C" int slpic_fp64_create(const slpic_config *c, slpic_fp64_t **out)
     if (e == cudaSuccess)
         e = cudaMemset(p.E, 0, sizeof(double) * nn);
     if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(k_step64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+        e = slpic::allow_dynamic_smem(k_step64, smem);
     int occ = 0;
     if (e == cudaSuccess)
         e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k_step64, kThreads, smem);

@@ -59,3 +59,18 @@ def test_batch_with_a_smaller_batch_beside_it(cells):
     for ps, st, mine in zip(probs, states, got):
         for a, b in zip(mine, _batch_run(binding.Batch(ps), ps, st)):
             assert np.array_equal(a, b)
+
+
+def test_fp64_form_with_a_smaller_grid_beside_it():
+    probs = [inputs.sheath_problem(n_cells=n, ppc=4, v0=0.1) for n in (9000, 64)]
+    states = [inputs.load_state(p) for p in probs]
+    sims = [binding.SimulationFP64(p) for p in probs]
+    for sim, prob, state in zip(sims, probs, states):
+        for s, st in enumerate(state):
+            sim.load_cells(s, *st)
+        sim.prepare()
+        sim.step(3)
+        rho = sim.fields()[0]
+        assert np.isfinite(rho).all() and rho.size == prob["n_cells"] + 1
+        assert sum(sim.count(s) for s in range(2)) > 0
+        sim.close()
