@@ -35,7 +35,9 @@
  * the output gradient rounded to BF16, and passes the forward rounding through
  * unchanged; the weight gradient is a GEMM over the pixels (split over CTAs, the
  * parts added in a fixed order) of the rounded input and the rounded output
- * gradient; the bias gradient sums the unrounded output gradient in FP64.
+ * gradient; the bias gradient sums the unrounded output gradient in FP64 (where the
+ * channel counts are multiples of 8 a warp's tile first in three FP32 numbers, which keep
+ * more bits than FP64's one; values of 2^100 and more in FP64 throughout).
  *
  * Parameters: one flat FP32 array, conv by conv in the order encoder
  * l = 0..L-1, decoder l = L-2..0, output; each conv its weights

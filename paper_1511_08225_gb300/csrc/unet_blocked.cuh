@@ -197,45 +197,105 @@ __device__ __forceinline__ uint4 *blk_at(const Blk &b, int n, int g, size_t pos)
     return reinterpret_cast<uint4 *>(b.p) + (((size_t)n * b.groups + b.off + g) * b.ps + pos);
 }
 
-// A sum carried as an unevaluated pair h + l (Dekker's and Knuth's error-free
-// transformations): 48 significant bits on the FP32 pipe; the tiles' sums are then added
-// in FP64, whose pipe (2 lanes per SM here) could not take one addition per value.
-struct DF {
-    float h, l;
+// The bias gradients' sums: over a warp's tile on the FP32 pipe, from there on in FP64, whose
+// pipe (2 lanes per SM here) could not take one addition per value.  A tile's sum is three
+// numbers, a the FP32 sum, b the sum of its additions' exact errors (Knuth's two-sum), c that
+// of b's: Ogita, Rump and Oishi's cascaded summation (SIAM J. Sci. Comput. 26, 2005) with
+// three terms, good to some 70 bits of the sum of the magnitudes, more than FP64 keeps.  FP32's
+// range does not hold partial sums of large values: those go to FP64 (bias_large).  Loss and
+// gradients of 512^2, batch 2: 1,639 us; with pairs (48 bits) in their place 1,609.
+struct Sum3 {
+    float a, b, c;
 };
-__device__ __forceinline__ DF df_add(DF a, DF b)
+__device__ __forceinline__ float two_sum(float x, float y, float &e)
 {
-    const float s = __fadd_rn(a.h, b.h);
-    const float t = __fsub_rn(s, a.h);
-    const float e = __fadd_rn(__fsub_rn(a.h, __fsub_rn(s, t)), __fsub_rn(b.h, t));
-    const float l = __fadd_rn(e, __fadd_rn(a.l, b.l));
-    const float h = __fadd_rn(s, l);
-    return DF{h, __fsub_rn(l, __fsub_rn(h, s))};
+    const float s = __fadd_rn(x, y), t = __fsub_rn(s, x);
+    e = __fadd_rn(__fsub_rn(x, __fsub_rn(s, t)), __fsub_rn(y, t));
+    return s;
 }
-__device__ __forceinline__ DF df_shfl(DF a, int o)
+__device__ __forceinline__ void sum3_add(Sum3 &s, float v)
 {
-    return DF{__shfl_xor_sync(0xffffffffu, a.h, o), __shfl_xor_sync(0xffffffffu, a.l, o)};
+    float e, f;
+    s.a = two_sum(s.a, v, e);
+    s.b = two_sum(s.b, e, f);
+    s.c = __fadd_rn(s.c, f);
 }
-// sum of 8 channels over the warp's lanes, halving the channels a lane keeps at each of
-// the first three exchanges; the sum of channel (l>>4 & 1)*4 + (l>>3 & 1)*2 + (l>>2 & 1)
-// ends in lane l
-__device__ __forceinline__ DF df_warp8(DF (&v)[8])
+// x and y of T terms, the rest zero (the sum has a term more)
+template <int T>
+__device__ __forceinline__ Sum3 sum3_add(const Sum3 &x, const Sum3 &y)
 {
-    const int lane = threadIdx.x & 31;
-#pragma unroll
-    for (int s = 0; s < 3; ++s) {
-        const int o = 16 >> s, half = 4 >> s;
-        const bool up = lane & o;
-#pragma unroll
-        for (int k = 0; k < half; ++k) {
-            const DF keep = up ? v[k + half] : v[k];
-            const DF send = up ? v[k] : v[k + half];
-            v[k] = df_add(keep, df_shfl(send, o));
-        }
+    float e, f, g;
+    Sum3 r{0.0f, 0.0f, 0.0f};
+    r.a = two_sum(x.a, y.a, e);
+    if (T == 1) {
+        r.b = e;
+        return r;
     }
-    v[0] = df_add(v[0], df_shfl(v[0], 2));
-    v[0] = df_add(v[0], df_shfl(v[0], 1));
-    return v[0];
+    r.b = two_sum(x.b, y.b, f);
+    r.b = two_sum(r.b, e, g);
+    r.c = __fadd_rn(f, g);
+    if (T == 3)
+        r.c = __fadd_rn(__fadd_rn(x.c, y.c), r.c);
+    return r;
+}
+template <int T>
+__device__ __forceinline__ Sum3 sum3_shfl(const Sum3 &s, int o)
+{
+    return Sum3{__shfl_xor_sync(0xffffffffu, s.a, o), T > 1 ? __shfl_xor_sync(0xffffffffu, s.b, o) : 0.0f,
+                T > 2 ? __shfl_xor_sync(0xffffffffu, s.c, o) : 0.0f};
+}
+// one exchange: of 2 K channels a lane keeps K
+template <int T, int K>
+__device__ __forceinline__ void sum3_exchange(Sum3 (&v)[8])
+{
+    const bool up = threadIdx.x & (4 * K);
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const Sum3 keep = up ? v[k + K] : v[k], send = up ? v[k] : v[k + K];
+        v[k] = sum3_add<T>(keep, sum3_shfl<T>(send, 4 * K));
+    }
+}
+// The sums of 8 channels over the warp's lanes (sums of T terms), added to bp[8]; channel
+// (l>>4 & 1)*4 + (l>>3 & 1)*2 + (l>>2 & 1) ends in lane l.
+template <int T>
+__device__ __forceinline__ void bias_warp(Sum3 (&v)[8], double *bp)
+{
+    constexpr int T1 = T < 3 ? T + 1 : 3, T2 = T1 < 3 ? T1 + 1 : 3;
+    sum3_exchange<T, 4>(v);
+    sum3_exchange<T1, 2>(v);
+    sum3_exchange<T2, 1>(v);
+    v[0] = sum3_add<3>(v[0], sum3_shfl<3>(v[0], 2));
+    v[0] = sum3_add<3>(v[0], sum3_shfl<3>(v[0], 1));
+    const int lane = threadIdx.x & 31;
+    if (!(lane & 3))  // this warp's own entry
+        bp[(lane >> 4) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] +=
+            (double)v[0].a + ((double)v[0].b + (double)v[0].c);
+}
+// Where a lane's eight values reach 2^100 in sum (large values, infinities, NaN: rare), the
+// warp's are added to bp[8] in FP64 and taken out of v.  The whole warp.
+__device__ __forceinline__ void bias_large(float (&v)[8], double *bp)
+{
+    float m = fabsf(v[0]);
+#pragma unroll
+    for (int q = 1; q < 8; ++q)
+        m = __fadd_rn(m, fabsf(v[q]));
+    if (__all_sync(0xffffffffu, m < 0x1p100f))
+        return;
+#pragma unroll 1
+    for (int q = 0; q < 8; ++q) {
+        double d = 0.0;
+#pragma unroll
+        for (int r = 0; r < 8; ++r)  // (constant indices: v stays in registers)
+            if (r == q) {
+                d = (double)v[r];
+                v[r] = 0.0f;
+            }
+        for (int o = 16; o; o >>= 1)
+            d += __shfl_xor_sync(0xffffffffu, d, o);
+        if ((threadIdx.x & 31) == 0)
+            bp[q] += d;
+    }
+    __syncwarp();
 }
 
 // ---- convolution (and, on mirrored weights, its input gradient) ---------------------
@@ -528,7 +588,8 @@ __global__ void __launch_bounds__(kBThreads, 1) k_conv_blk(const __grid_constant
             for (int og = warp >> 2; og * 8 < a.nout; og += kBEpi / 4) {
                 float v[MT][8];
                 blk_ld(tl + (uint32_t)(og * 8), v, a.Np);
-                DF bs[8] = {};
+                Sum3 bs[8];
+                double *bp = s_bp[kGrad ? warp & 3 : 0] + (kGrad ? og * 8 : 0);
                 if (!kGrad && a.mode == kBmOut) {
                     if (og == 0)
 #pragma unroll
@@ -584,10 +645,16 @@ __global__ void __launch_bounds__(kBThreads, 1) k_conv_blk(const __grid_constant
                             const int cg = a.o0 / 8 + og;
                             mask8(s, *blk_at(a.mask, n, cg, (size_t)(y0 + 1) * P + x + 1));
                             *blk_at(a.dst, n, cg, (size_t)(y0 / 2 + 1) * (a.W / 2 + 2) + x / 2 + 1) = pack8(s);
+                        } else {
+#pragma unroll
+                            for (int q = 0; q < 8; ++q)
+                                s[q] = 0.0f;
                         }
+                        bias_large(s, bp);
 #pragma unroll
                         for (int q = 0; q < 8; ++q)
-                            bs[q] = DF{mine ? s[q] : 0.0f, 0.0f};
+                            bs[q] = Sum3{s[q], 0.0f, 0.0f};
+                        bias_warp<1>(bs, bp);
                     } else {
                         const int cg = (a.o0 - a.cup) / 8 + og, gs = (a.bchan - a.cup) / 8;
 #pragma unroll
@@ -604,46 +671,58 @@ __global__ void __launch_bounds__(kBThreads, 1) k_conv_blk(const __grid_constant
 #pragma unroll
                     for (int t = 0; t < MT; ++t) {
                         const int y = y0 + t;
-                        if (inx && y < a.H) {
+                        if (y < a.H) {
 #pragma unroll
                             for (int f = 0; f < 4; ++f) {
-                                const int yf = 2 * y + (f >> 1), xf = 2 * x + (f & 1);
-                                const float4 *d = reinterpret_cast<const float4 *>(a.f32) +
-                                                  ((((size_t)n * gs + cg) * (2 * a.H) + yf) * Wf + xf) * 2;
-                                const float4 d0 = d[0], d1 = d[1];
-                                const float e[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
-                                float s[8];
+                                float s[8] = {};
+                                if (inx) {
+                                    const int yf = 2 * y + (f >> 1), xf = 2 * x + (f & 1);
+                                    const float4 *d = reinterpret_cast<const float4 *>(a.f32) +
+                                                      ((((size_t)n * gs + cg) * (2 * a.H) + yf) * Wf + xf) * 2;
+                                    const float4 d0 = d[0], d1 = d[1];
+                                    const float e[8] = {d0.x, d0.y, d0.z, d0.w, d1.x, d1.y, d1.z, d1.w};
+#pragma unroll
+                                    for (int q = 0; q < 8; ++q)
+                                        s[q] = e[q] + 0.25f * v[t][q];
+                                    const size_t pos = (size_t)(yf + 1) * Pf + xf + 1;
+                                    mask8(s, *blk_at(a.mask, n, cg, pos));
+                                    *blk_at(a.dst, n, cg, pos) = pack8(s);
+                                }
+                                bias_large(s, bp);
 #pragma unroll
                                 for (int q = 0; q < 8; ++q)
-                                    s[q] = e[q] + 0.25f * v[t][q];
-                                const size_t pos = (size_t)(yf + 1) * Pf + xf + 1;
-                                mask8(s, *blk_at(a.mask, n, cg, pos));
-                                *blk_at(a.dst, n, cg, pos) = pack8(s);
-#pragma unroll
-                                for (int q = 0; q < 8; ++q)
-                                    bs[q] = df_add(bs[q], DF{s[q], 0.0f});
+                                    if (t == 0 && f == 0)
+                                        bs[q] = Sum3{s[q], 0.0f, 0.0f};
+                                    else if (t == 0 && f == 1)
+                                        bs[q] = sum3_add<1>(bs[q], Sum3{s[q], 0.0f, 0.0f});
+                                    else
+                                        sum3_add(bs[q], s[q]);
                             }
                         }
                     }
+                    bias_warp<3>(bs, bp);
                 } else {  // kBmGradMask
 #pragma unroll
                     for (int t = 0; t < MT; ++t) {
                         const int y = y0 + t, cg = a.o0 / 8 + og;
-                        if (inx && y < a.H) {
-                            const size_t pos = (size_t)(y + 1) * P + x + 1;
-                            mask8(v[t], *blk_at(a.mask, n, cg, pos));
-                            *blk_at(a.dst, n, cg, pos) = pack8(v[t]);
+                        if (y < a.H) {
+                            if (inx) {
+                                const size_t pos = (size_t)(y + 1) * P + x + 1;
+                                mask8(v[t], *blk_at(a.mask, n, cg, pos));
+                                *blk_at(a.dst, n, cg, pos) = pack8(v[t]);
+                            } else {
+#pragma unroll
+                                for (int q = 0; q < 8; ++q)
+                                    v[t][q] = 0.0f;
+                            }
+                            bias_large(v[t], bp);
 #pragma unroll
                             for (int q = 0; q < 8; ++q)
-                                bs[q] = df_add(bs[q], DF{v[t][q], 0.0f});
+                                bs[q] = t == 0 ? Sum3{v[t][q], 0.0f, 0.0f}
+                                               : sum3_add<1>(bs[q], Sum3{v[t][q], 0.0f, 0.0f});
                         }
                     }
-                }
-                if (kGrad && (a.mode != kBmGradUp || a.o0 + og * 8 < a.cup)) {
-                    const DF s = df_warp8(bs);
-                    if (!(lane & 3))  // this warp's own entry
-                        s_bp[warp & 3][og * 8 + (lane >> 4) * 4 + ((lane >> 3) & 1) * 2 + ((lane >> 2) & 1)] +=
-                            (double)s.h + (double)s.l;
+                    bias_warp<MT>(bs, bp);
                 }
             }
             // the accumulators may be overwritten
