@@ -203,7 +203,10 @@ int slpic_prepare(slpic_t *h);
  * pushed next step) and solve phi^{n+1}, E^{n+1}.  The steps run as a
  * captured CUDA graph with no host synchronisation between them; a call of 4 or
  * more steps of a simulation of at most 7 million slots (capacities) runs them
- * in one launch instead (at most 4096 steps each), with the same results. */
+ * in one launch instead (at most 4096 steps each), with the same results, unless
+ * the grid leaves it no room in shared memory (beyond some 8,500 nodes with two
+ * species), the field is a prescribed wave, kernel timing is on, or the tuning asks
+ * for the per-warp particle kernel. */
 int slpic_step(slpic_t *h, int64_t nsteps);
 
 /* Wait for queued work; report device-side errors raised since the last
@@ -285,11 +288,15 @@ int slpic_kernel_times(slpic_t *h, double *particle_ms, double *hard_ms, double 
  * skips its remaining tiles, waits for its own copies still in flight (with the
  * default limit, whatever `cycles` is) and returns, so the GPU context stays
  * usable.  The step it cut short leaves the handle's particles and fields no longer
- * those of the method: destroy the handle (reading it back stays safe).  A limit far
- * below a copy's latency exercises that path.  Below the default the waits poll the
- * barrier without suspending the thread (which costs issue slots), so that a short
- * limit can run out.  Takes effect from the next step (the step graphs are captured
- * again).  SLPIC_ERR_INVALID for cycles < 0 or a batch. */
+ * those of the method: destroy the handle (reading it back stays safe).  The limit also
+ * bounds the thread blocks' wait for one another where many steps run in one launch
+ * (slpic_step): then all of them leave at the end of the same whole step, launches
+ * queued behind make no step, and once the error has been reported the handle stands at
+ * that step, ready to go on.  A limit far below a copy's latency exercises these
+ * paths.  Below the default the particle kernel's waits poll the barrier without
+ * suspending the thread (which costs issue slots), so that a short limit can run out.
+ * Takes effect from the next step (the step graphs are captured again).
+ * SLPIC_ERR_INVALID for cycles < 0 or a batch. */
 int slpic_set_wait_limit(slpic_t *h, int64_t cycles);
 
 /* Device time of the step's kernels, always recorded: for kind 0 (the particle

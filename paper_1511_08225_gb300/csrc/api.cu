@@ -698,11 +698,10 @@ static int capture(slpic_t *h, long long first_step, int nsteps, bool timed,
 
 // Whether a call of nsteps steps runs in one launch (k_steps): a small simulation and more
 // than a few steps, none of the modes that k_steps does not have (the prescribed wave,
-// timed graphs, the per-warp kernel, a changed wait limit, which is the TMA kernel's).
+// timed graphs, the per-warp kernel).
 static bool steps_fused(const slpic_t *h, int64_t nsteps)
 {
-    return h->d_steps && nsteps >= kStepsFewest && !h->p.wave_on && h->t_len == 0 && h->particle_kernel == 0 &&
-           h->p.wait_cycles == kWaitCycles;
+    return h->d_steps && nsteps >= kStepsFewest && !h->p.wave_on && h->t_len == 0 && h->particle_kernel == 0;
 }
 
 extern "C" int slpic_step(slpic_t *h, int64_t nsteps)
@@ -793,7 +792,15 @@ static int wait_status(slpic_t *h, char *stage)
     std::memcpy(&e, stage, sizeof(e));
     if (e) {
         int zero = 0;
+        long long step = h->step;
         CK(h, cudaMemcpy(&h->d_state->error, &zero, sizeof(int), cudaMemcpyHostToDevice));
+        CK(h, cudaMemcpy(&step, &h->d_state->step, sizeof(step), cudaMemcpyDeviceToHost));
+        if (step != h->step) {
+            // k_steps was cut short: the handle stands where the device does, its deposit and
+            // field to be made from the particles there
+            h->step = step;
+            h->dirty = true;
+        }
         return fail(h, e, e == SLPIC_ERR_CAPACITY  ? "particle store full: injection truncated"
                           : e == SLPIC_ERR_TIMEOUT ? "a bounded wait of a particle or step kernel ran out"
                                                    : "device error");

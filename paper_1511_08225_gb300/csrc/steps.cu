@@ -56,9 +56,13 @@ size_t steps_smem_bytes(int nn, int ns, bool profile)
 
 __device__ __forceinline__ void steps_fence() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
 
-// All CTAs (co-resident: a cooperative launch), the k-th barrier of the launch; false after
-// about a second, recorded as SLPIC_ERR_TIMEOUT.
-__device__ __forceinline__ bool steps_barrier(StepsScratch *sc, unsigned target, int *error)
+// All CTAs (co-resident: a cooperative launch), once `target` have arrived in the launch.  A wait
+// longer than `limit` SM cycles ends the launch (SLPIC_ERR_TIMEOUT): the CTA that gives up marks
+// the counter, which it can only while one has not arrived, and nobody passes a marked
+// counter.  So the barrier has one outcome for all: true everywhere, or false everywhere.
+constexpr unsigned kStepsGivenUp = 0x80000000u;
+
+__device__ __forceinline__ bool steps_barrier(StepsScratch *sc, unsigned target, long long limit, int *error)
 {
     __shared__ int s_ok;
     __syncthreads();
@@ -70,10 +74,14 @@ __device__ __forceinline__ bool steps_barrier(StepsScratch *sc, unsigned target,
         int ok = 1;
         for (;;) {
             asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&sc->bar) : "memory");
+            if (v & kStepsGivenUp) {
+                ok = 0;
+                break;
+            }
             if (v >= target)
                 break;
-            if (clock64() - t0 > kWaitCycles) {
-                atomicCAS(error, 0, SLPIC_ERR_TIMEOUT);
+            if (clock64() - t0 > limit && atomicCAS(&sc->bar, v, v | kStepsGivenUp) == v) {
+                atomicExch(error, SLPIC_ERR_TIMEOUT);
                 ok = 0;
                 break;
             }
@@ -145,7 +153,8 @@ struct StepsShared {
     int cut;                                         // a source was truncated
     unsigned lost[kMaxSpecies][2];                   // absorbed by this CTA in this step
     unsigned listed;
-    unsigned long long iterative[kMaxSpecies];       // walked by this CTA
+    unsigned walked[kMaxSpecies];                    // by this CTA in this step
+    unsigned long long iterative[kMaxSpecies];       // ... in the launch's steps before
     unsigned long long part[kMaxSpecies][kSW][4];    // per warp: sums of R, W (two words), T
     unsigned long long tot[kMaxSpecies][4];
     double K[kMaxSpecies];                           // k_field's K_s
@@ -307,6 +316,8 @@ __global__ void __launch_bounds__(kST, 1)
     unsigned long long *acc3 = reinterpret_cast<unsigned long long *>(sc + 1);
     DevState *st = p.st;
     const long long step0 = *(volatile long long *)&st->step;
+    if (*(volatile int *)&st->error == SLPIC_ERR_TIMEOUT)
+        return;  // the launch before was cut short: no step until that has been reported
 
     for (int j = t; j < tot; j += kST) {
         s_lo[j] = 0u;
@@ -323,7 +334,7 @@ __global__ void __launch_bounds__(kST, 1)
         sh.holes[t] = t < ns ? (long long)*(volatile unsigned long long *)&st->holes[t][P] : 0;
         sh.frac[t] = t < ns ? *(volatile double *)&st->src_frac[t] : 0.0;
         sh.injected[t] = sh.absorbed[t][0] = sh.absorbed[t][1] = 0;
-        sh.iterative[t] = 0;
+        sh.iterative[t] = sh.walked[t] = 0;
         sh.K[t] = t < ns ? p.k2 * p.sp[t].rho_unit * (0.5 * p.inv_dx) : 0.0;
         sh.lost[t][0] = sh.lost[t][1] = 0u;
     }
@@ -340,8 +351,8 @@ __global__ void __launch_bounds__(kST, 1)
             tick = now;
         }
     };
-    int turn = 0;
-    for (int e = 0; e < nsteps; ++e) {
+    int turn = 0, e = 0;  // e: whole steps made
+    for (; e < nsteps; ++e) {
         const long long step = step0 + e;
         const int P = (int)(step & 1), Q = P ^ 1;
         const bool compact = step % every == every - 1, last = e + 1 == nsteps;
@@ -408,7 +419,7 @@ __global__ void __launch_bounds__(kST, 1)
                 unsigned b = 0;
                 if (lane == 0) {
                     b = atomicAdd(&sh.listed, (unsigned)__popc(hm));
-                    atomicAdd(&sh.iterative[s], (unsigned long long)__popc(hm));
+                    atomicAdd(&sh.walked[s], (unsigned)__popc(hm));
                 }
                 b = __shfl_sync(0xffffffffu, b, 0) + __popc(hm & ((1u << lane) - 1u));
                 if (hard) {
@@ -497,8 +508,8 @@ __global__ void __launch_bounds__(kST, 1)
         if (blockIdx.x == 0 && t < kMaxSpecies)
             sc->out[next][t] = sc->absorbed[next][t][0] = sc->absorbed[next][t][1] = 0ULL;
         lap(1);
-        if (!steps_barrier(sc, (unsigned)(e + 1) * gridDim.x, &st->error))
-            return;
+        if (!steps_barrier(sc, (unsigned)(e + 1) * gridDim.x, p.wait_cycles, &st->error))
+            break;
 
         // ---- the step's totals, and the source (thread s for species s; every CTA the same)
         if (t < ns) {
@@ -518,6 +529,8 @@ __global__ void __launch_bounds__(kST, 1)
             sh.make[t] = k;
             sh.count[t] = have + k;
             sh.holes[t] = compact ? 0 : sh.holes[t] + (long long)(a0 + a1);
+            sh.iterative[t] += sh.walked[t];
+            sh.walked[t] = 0u;
             sh.injected[t] += k;
             sh.absorbed[t][0] += (long long)a0;
             sh.absorbed[t][1] += (long long)a1;
@@ -588,11 +601,12 @@ __global__ void __launch_bounds__(kST, 1)
         lap(2);
         turn = next;
     }
-    // ---- the launch's bookkeeping
+    // ---- the launch's bookkeeping: of the whole steps (a step that was cut short has written
+    // only the other buffers; deposit and field are then made again on the host's demand)
     if (t < ns && sh.iterative[t])
         atomicAdd((unsigned long long *)&st->iterative_total[t], sh.iterative[t]);
     if (blockIdx.x == 0 && t < ns) {
-        const int Pf = (int)((step0 + nsteps) & 1);
+        const int Pf = (int)((step0 + e) & 1);
         st->count[t][Pf] = (unsigned long long)sh.count[t];
         st->holes[t][Pf] = (unsigned long long)sh.holes[t];
         st->count[t][Pf ^ 1] = 0ULL;
@@ -607,9 +621,9 @@ __global__ void __launch_bounds__(kST, 1)
             atomicCAS(&st->error, 0, SLPIC_ERR_CAPACITY);
         for (int k = 0; k < 3; ++k) {
             st->span_ns[k] += span[k];
-            st->span_launches[k] += (unsigned long long)nsteps;
+            st->span_launches[k] += (unsigned long long)e;
         }
-        st->step = step0 + nsteps;
+        st->step = step0 + e;
     }
 }
 
