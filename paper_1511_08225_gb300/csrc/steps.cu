@@ -5,12 +5,12 @@
 // round trips between them.  Here one cooperative launch runs the steps.  Every CTA (one
 // per SM, leaving one SM free for overlapped read-backs) pushes its share of the slots as
 // k_particles does, walks the pushes that need iteration from a list of its own in shared
-// memory, and adds its charge to a global accumulator; then comes the step's only grid
-// barrier; then every CTA makes the field for itself: it reads the summed deposit, adds
-// the source particles' (made from their counters by every CTA, and stored by the one
-// that pushes them next) and solves for E as k_field does, with the
-// same integers and the same FP64 operations.  Nothing else of a step crosses CTAs, so
-// 256 cells and 51,200 particles step in 9 us, 100 cells and 1.4e5 in 11.
+// memory, and adds its charge to a global accumulator; then comes the step's grid barrier;
+// then every CTA makes the field for itself: it reads the summed deposit, adds the source
+// particles' (made from their counters by every CTA, and stored by the one that pushes them
+// next; a large source is made in shares and has a barrier of its own) and solves for E as
+// k_field does, with the same integers and the same FP64 operations.  Nothing else of a step
+// crosses CTAs, so 256 cells and 51,200 particles step in 12 us, 100 cells and 1.4e5 in 13.
 //
 // Particles, deposits, fields and counters are those of the three kernels bit for bit.
 // The accumulators, the absorbed counts and a compacting step's output counts go by three
@@ -29,6 +29,12 @@ namespace slpic {
 constexpr int kST = kStepsThreads;
 constexpr int kSW = kST / 32;
 constexpr int kSList = 512;  // listed iterative pushes of a CTA and step (more are pushed in place)
+// Source particles of a step that every CTA makes for itself; more are made in shares, which
+// costs another barrier (4 us) and saves 1.6 us per 1,000 particles.  us a step, every CTA all of
+// them / in shares / the three kernels, two species of 1,000, 2,000, 10,000 and 100,000 each:
+// 256 cells 27 / 27 / 39, 33 / 28 / 44, 83 / 45 / 93, 575 / 172 / 749; 4,096 cells 30 / 30 / 38,
+// 35 / 30 / 39, 77 / 40 / 55, 510 / 109 / 329; a wall source of 300 14 / 17 / 33.
+constexpr int kStepsOwnSource = 2048;
 
 struct StepsScratch {
     unsigned bar;  // arrivals at the grid barrier
@@ -151,6 +157,11 @@ struct StepsShared {
     double frac[kMaxSpecies];
     long long base[kMaxSpecies], make[kMaxSpecies];  // this step's source: first slot, particles
     int cut;                                         // a source was truncated
+    struct Counts {  // before this step, and what it has absorbed and walked
+        long long count, holes, lo, hi;
+        double frac;
+        unsigned walked;
+    } before[kMaxSpecies];
     unsigned lost[kMaxSpecies][2];                   // absorbed by this CTA in this step
     unsigned listed;
     unsigned walked[kMaxSpecies];                    // by this CTA in this step
@@ -351,7 +362,8 @@ __global__ void __launch_bounds__(kST, 1)
             tick = now;
         }
     };
-    int turn = 0, e = 0;  // e: whole steps made
+    int turn = 0, e = 0;      // e: whole steps made
+    unsigned arrivals = 0u;  // of all CTAs at the barriers so far
     for (; e < nsteps; ++e) {
         const long long step = step0 + e;
         const int P = (int)(step & 1), Q = P ^ 1;
@@ -508,10 +520,12 @@ __global__ void __launch_bounds__(kST, 1)
         if (blockIdx.x == 0 && t < kMaxSpecies)
             sc->out[next][t] = sc->absorbed[next][t][0] = sc->absorbed[next][t][1] = 0ULL;
         lap(1);
-        if (!steps_barrier(sc, (unsigned)(e + 1) * gridDim.x, p.wait_cycles, &st->error))
+        arrivals += gridDim.x;
+        if (!steps_barrier(sc, arrivals, p.wait_cycles, &st->error))
             break;
 
-        // ---- the step's totals, and the source (thread s for species s; every CTA the same)
+        // ---- the step's totals and the source's counts (thread s for species s; every CTA the
+        // same)
         if (t < ns) {
             const unsigned long long a0 = __ldcg(&sc->absorbed[turn][t][0]), a1 = __ldcg(&sc->absorbed[turn][t][1]);
             const unsigned long long ref =
@@ -520,6 +534,8 @@ __global__ void __launch_bounds__(kST, 1)
             double f = sh.frac[t];
             long long k = source_count(p, p.sp[t], ref, f);
             const long long room = p.sp[t].capacity - have;
+            sh.before[t] = StepsShared::Counts{sh.count[t], sh.holes[t], (long long)a0, (long long)a1, sh.frac[t],
+                                               sh.walked[t]};
             if (k > room) {
                 k = room;
                 sh.cut = 1;
@@ -538,13 +554,24 @@ __global__ void __launch_bounds__(kST, 1)
         for (int j = t; j < tot; j += kST)
             s_acc[j] = __ldcg(acc3 + (size_t)turn * tot + j);
         __syncthreads();
+        // ---- the source's particles: few are made by every CTA, more in shares, with their
+        // charge through the accumulator and a barrier of its own
         {
             long long pre[kMaxSpecies + 1];
             pre[0] = 0;
 #pragma unroll
             for (int s = 0; s < kMaxSpecies; ++s)
                 pre[s + 1] = pre[s] + (s < ns ? sh.make[s] : 0);
-            for (long long k = t; k < pre[kMaxSpecies]; k += kST) {
+            const bool shares = pre[kMaxSpecies] > kStepsOwnSource;
+            long long k = t, k1 = pre[kMaxSpecies];
+            if (shares) {
+                k = t + k1 * blockIdx.x / gridDim.x;
+                k1 = k1 * (blockIdx.x + 1) / gridDim.x;
+                for (int j = t; j < tot; j += kST)
+                    s_acc[j] = 0ULL;
+                __syncthreads();
+            }
+            for (; k < k1; k += kST) {
                 int s = 0;
                 long long i = k;
 #pragma unroll
@@ -575,10 +602,32 @@ __global__ void __launch_bounds__(kST, 1)
                 if (rhi)
                     atomicAdd(acc + 2 * c1 + 1, rhi);
                 const int o = (int)(sh.base[s] + i);  // stored by the CTA that pushes it next
-                if ((o >> 5) % (int)gridDim.x == steps_first_tile(s)) {
+                if (shares || (o >> 5) % (int)gridDim.x == steps_first_tile(s)) {
                     sp.cell[Q][o] = c;
                     sp.pv[Q][o] = q;
                 }
+            }
+            if (shares) {
+                __syncthreads();
+                for (int j = t; j < tot; j += kST)
+                    if (s_acc[j])
+                        atomicAdd(acc3 + (size_t)turn * tot + j, s_acc[j]);
+                arrivals += gridDim.x;
+                if (!steps_barrier(sc, arrivals, p.wait_cycles, &st->error)) {
+                    if (t < ns) {  // the step is not whole: its counts taken back
+                        const StepsShared::Counts &c = sh.before[t];
+                        sh.count[t] = c.count;
+                        sh.holes[t] = c.holes;
+                        sh.frac[t] = c.frac;
+                        sh.iterative[t] -= c.walked;
+                        sh.injected[t] -= sh.make[t];
+                        sh.absorbed[t][0] -= c.lo;
+                        sh.absorbed[t][1] -= c.hi;
+                    }
+                    break;
+                }
+                for (int j = t; j < tot; j += kST)
+                    s_acc[j] = __ldcg(acc3 + (size_t)turn * tot + j);
             }
         }
         __syncthreads();
