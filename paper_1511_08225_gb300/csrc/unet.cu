@@ -1279,7 +1279,11 @@ WgPlan wg_plan(const slpic_unet_t *h, const ConvSpec &c, int Np, int nb)
     q.gx = (q.mtiles + q.mper - 1) / q.mper;
     q.gy = q.djs == 3 ? 1 : 3;
     const long long chunks = (long long)nb * (((long long)hl(h, c.level) * (wl(h, c.level) + 2) + kWKP - 1) / kWKP);
-    q.splits = (int)std::max(1LL, std::min(chunks, (long long)152 / (q.gx * q.gy)));
+    // a wave of CTAs; two waves' worth of (dj, tile) pairs where the tiles do not fill the
+    // CTAs (128 -> 256 channels: 33 ranges, not 25, for 20 us of 1,640 at 512^2, batch 2), so
+    // that no range's FP32 sum is longer than the gather kernel's
+    const int most = std::max(152 / (q.gx * q.gy), 2 * 152 / (3 * q.mtiles));
+    q.splits = (int)std::max(1LL, std::min(chunks, (long long)most));
     return q;
 }
 
