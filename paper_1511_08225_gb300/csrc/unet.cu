@@ -780,6 +780,49 @@ __global__ void __launch_bounds__(kT) k_norm_apply(const float *__restrict__ x, 
         xs[o + q] = x[o + q] * inv;
 }
 
+// All of it in one launch, a CTA per sample (xs null: the scale alone): small images, where the
+// launches cost more than the sum on one SM's FP64 pipe (two operations a pixel on 2 lanes).
+// A forward pass in FP32, us, one launch / three: 64^2 82 / 86, 80^2 84 / 87, 96^2 86 / 87,
+// 128^2 90 / 86; with tensor cores 48 / 49, 49 / 51, 51 / 51, 55 / 51.
+constexpr int kNormOneThreads = 1024;
+constexpr size_t kNormOne = 8192;  // most pixels of a sample
+
+__global__ void __launch_bounds__(kNormOneThreads) k_norm_one(const float *__restrict__ x,
+                                                            float *__restrict__ xs, float *__restrict__ s,
+                                                            int HW, int normalise)
+{
+    __shared__ double s_red[kNormOneThreads / 32];
+    __shared__ float s_scale;
+    const size_t o = (size_t)blockIdx.x * HW;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    double acc = 0.0;
+    if (normalise)
+        for (int q = threadIdx.x; q < HW; q += kNormOneThreads) {
+            const double v = x[o + q];
+            acc = fma(v, v, acc);  // (the square of a float is exact in FP64)
+        }
+    for (int off = 16; off; off >>= 1)
+        acc += __shfl_down_sync(0xffffffffu, acc, off);
+    if (lane == 0)
+        s_red[warp] = acc;
+    __syncthreads();
+    if (warp == 0) {
+        double v = lane < (int)(blockDim.x >> 5) ? s_red[lane] : 0.0;
+        for (int off = 16; off; off >>= 1)
+            v += __shfl_down_sync(0xffffffffu, v, off);
+        if (lane == 0) {
+            const float sc = normalise ? (float)sqrt(v / (double)HW) : 1.0f;
+            s_scale = s[blockIdx.x] = sc > 0.0f ? sc : 1.0f;
+        }
+    }
+    if (!xs)
+        return;
+    __syncthreads();
+    const float inv = 1.0f / s_scale;
+    for (int q = threadIdx.x; q < HW; q += kNormOneThreads)
+        xs[o + q] = x[o + q] * inv;
+}
+
 // y = y_net * s_n * out_scale
 __global__ void k_scale_out(const float *__restrict__ ynet, float *__restrict__ y,
                             const float *__restrict__ s, float out_scale, size_t HW, int nb)
@@ -1363,6 +1406,12 @@ void backward_blk(slpic_unet_t *h, int nb, cudaStream_t st)
 void normalise_in(slpic_unet_t *h, int nb, const float *x, cudaStream_t st)
 {
     const size_t HW = hwl(h, 0);
+    if (HW <= kNormOne) {
+        // (fewer threads than kNormOneThreads only where they take a pixel each)
+        const int threads = (int)std::min<size_t>((HW + 31) / 32 * 32, kNormOneThreads);
+        k_norm_one<<<nb, threads, 0, st>>>(x, h->blk ? nullptr : h->xin, h->s, (int)HW, h->cfg.normalise);
+        return;
+    }
     if (h->cfg.normalise)
         k_norm_sum<<<dim3(kNormCtas, (unsigned)nb), kT, 0, st>>>(x, HW, h->npart);
     k_norm_scale<<<nb, 32, 0, st>>>(h->npart, h->s, HW, h->cfg.normalise);
