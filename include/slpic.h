@@ -202,11 +202,11 @@ int slpic_prepare(slpic_t *h);
  * rho^{n+1}; then inject source particles (deposited into rho^{n+1}, first
  * pushed next step) and solve phi^{n+1}, E^{n+1}.  The steps run as a
  * captured CUDA graph with no host synchronisation between them; a call of 4 or
- * more steps of a simulation of at most 7 million slots (capacities) runs them
- * in one launch instead (at most 4096 steps each), with the same results, unless
- * the grid leaves it no room in shared memory (beyond some 8,500 nodes with two
- * species), the field is a prescribed wave, kernel timing is on, or the tuning asks
- * for the per-warp particle kernel. */
+ * more steps of a simulation of at most 7 million slots (capacities; fewer on
+ * periodic grids of more than 2,900 nodes) runs them in one launch instead (at most
+ * 4096 steps each), with the same results, unless the grid leaves it no room in shared
+ * memory (beyond some 8,500 nodes with two species), the field is a prescribed wave,
+ * kernel timing is on, or the tuning asks for the per-warp particle kernel. */
 int slpic_step(slpic_t *h, int64_t nsteps);
 
 /* Wait for queued work; report device-side errors raised since the last

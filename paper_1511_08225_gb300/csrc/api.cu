@@ -390,13 +390,11 @@ extern "C" int slpic_create(const slpic_config *cfg, slpic_t **out)
     CKC(configure_particles_tma(nn, &h->tma_stages));
     // small simulations: many steps in one launch (k_steps)
     {
-        long long slots = 0, most = 0;
-        for (int s = 0; s < ns; ++s) {
+        long long slots = 0;
+        for (int s = 0; s < ns; ++s)
             slots += cfg->species[s].capacity;
-            most = std::max(most, (long long)cfg->species[s].capacity);
-        }
         CKC(configure_steps(&h->steps_smem));
-        if (slots <= kStepsMaxSlots && most <= kStepsMaxSpecies &&
+        if (slots <= steps_max_slots(nn, cfg->bc == SLPIC_BC_PERIODIC) &&
             steps_smem_bytes(nn, ns, true) <= (size_t)h->steps_smem) {
             CKC(cudaMalloc(&h->d_steps, steps_scratch_bytes(nn, ns)));
             // a CTA per SM (one SM left free, as for the TMA kernel), fewer where that

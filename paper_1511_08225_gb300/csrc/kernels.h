@@ -43,8 +43,18 @@ constexpr int kStepsThreads = 1024;
 // Where the line lies (us a step, three kernels against k_steps): 2,560 particles 27 / 9,
 // 51,200 30 / 12, 5.2e5 42 / 25, 2.0e6 62 / 47, 4.9e6 83 / 75, 8.1e6 104 / 107.5.  The host
 // knows the slots, of which a third to all are in use: at 7e6 it is no slower for any count.
-constexpr long long kStepsMaxSlots = 7000000;         // most slots, all species
-constexpr long long kStepsMaxSpecies = (1LL << 24) - 1;  // ... and of one: its sums fit 64 bits
+// (A species' sums also have to fit 64 bits: fewer than 2^24 particles.)
+constexpr long long kStepsMaxSlots = 7000000;  // most slots, all species
+static_assert(kStepsMaxSlots < (1LL << 24), "steps_field");
+// Every CTA does the whole field, which the cheaper steps of a periodic grid (no walls, no
+// source, every slot in use) do not hide on many nodes (beta = 1: 3,000 nodes 6.9e6 81 / 83;
+// 4,000 5.0e6 72 / 69, 6.9e6 84 / 85; 6,000 3.5e6 62 / 61, 5.0e6 72 / 75; 8,400 1.0e6 46 / 46,
+// 2.0e6 53 / 56; between plates it holds at 8,400 and 6.9e6), so there the line comes down.
+constexpr long long steps_max_slots(int nn, bool periodic)
+{
+    const long long line = 1150LL * (9000 - nn);
+    return periodic && line < kStepsMaxSlots ? line : kStepsMaxSlots;
+}
 constexpr int kStepsFewest = 4, kStepsMost = 4096;  // steps of a launch
 size_t steps_scratch_bytes(int nn, int ns);
 size_t steps_smem_bytes(int nn, int ns, bool profile);
