@@ -206,7 +206,12 @@ int slpic_prepare(slpic_t *h);
  * periodic grids of more than 2,900 nodes) runs them in one launch instead (at most
  * 4096 steps each), with the same results, unless the grid leaves it no room in shared
  * memory (beyond some 8,500 nodes with two species), the field is a prescribed wave,
- * kernel timing is on, or the tuning asks for the per-warp particle kernel. */
+ * kernel timing is on, or the tuning asks for the per-warp particle kernel.  Such a
+ * launch holds its share of the GPU (a thread block of 1,024 threads for every 768
+ * slots, at most one on all SMs but one) until its steps are done: simulations that
+ * fill the GPU, stepped side by side on streams of their own, run one after another,
+ * and from four of them on calls of up to 3 steps, or a batch (slpic_create_batch),
+ * get more done. */
 int slpic_step(slpic_t *h, int64_t nsteps);
 
 /* Wait for queued work; report device-side errors raised since the last

@@ -1493,8 +1493,9 @@ extern "C" int slpic_create_batch(const slpic_config *cfgs, int m, slpic_t **out
 }
 
 // Work items of the batched particle kernels: the (instance, species) pairs' particles laid
-// end to end and cut into as many equal parts as there are CTAs (`waves` full waves of the
-// GPU, fewer if the parts would be smaller than `min_share`, but at least one CTA a pair).
+// end to end and cut into as many equal parts as there are CTAs: `waves` full waves of the
+// GPU, or where the parts would be smaller than `min_share` as few as make them that large or
+// one a pair, if that is more.
 static int batch_tables(slpic_t *h)
 {
     std::vector<int2> pair;           // instance, species

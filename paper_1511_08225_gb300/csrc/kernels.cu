@@ -757,7 +757,6 @@ __global__ void __launch_bounds__(kPB, 4) k_particles(const __grid_constant__ St
     span_exit(p.st, 0);
 }
 
-// Batched forms: CTA b works on (instance, species, share, shares) = work[b].
 // Batched: CTA b walks work items first[b] .. first[b+1]-1, each {instance, species, f0, f1}: the
 // instance's tiles of that species from f0 to f1 of kBatchParts.  The items are cut so that
 // every CTA has the same number of particles, whatever the instances' sizes; one CTA per item of

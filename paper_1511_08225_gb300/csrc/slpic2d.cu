@@ -1139,10 +1139,11 @@ __device__ __forceinline__ double cg_double(float x)
 }
 
 // (float)(a / b), the FP64 quotient rounded to FP32, without the FP64 division's chain of
-// some 15 dependent instructions: the significands as pairs of floats, a quotient with a
-// correction good to 2^-43, rounded; the FP64 division where that lies within 2^-38 of
-// the middle between two floats (one quotient in 2^13), or where the operands or the
-// quotient leave the normal range.
+// some 15 dependent instructions: the significands as pairs of floats and Dekker's quotient of
+// such pairs (Numer. Math. 18, 1971: a first quotient, corrected by its remainder, which a
+// fused multiply-add leaves exact), good to 2^-43, rounded; the FP64 division where that lies
+// within 2^-38 of the middle between two floats (one quotient in 2^13), or where the operands
+// or the quotient leave the normal range.
 __device__ __forceinline__ float cg_quotient(double a, double b)
 {
     const unsigned ah = (unsigned)__double2hiint(a), al = (unsigned)__double2loint(a);

@@ -1,4 +1,4 @@
-// steps.cu -- many timesteps of a small 1D simulation in one launch.
+// steps.cu -- many timesteps of a 1D simulation in one launch, up to some 7 million slots.
 //
 // A step of the three kernels of kernels.cu takes 28 us however few particles there are:
 // launches, the ramp of a one-CTA-per-SM grid, a cluster launch for the field, and global
